@@ -7,29 +7,44 @@
 // key) pairs at 4 D flops each: a compute-bound product, unlike the
 // memory-bound decoding kernels.  Both products run on the tensor cores:
 //   S = Q K^T   : M = 128 positions, N = 128 keys, K = D, operands in shared memory
-//   O += P V    : M = 128, N = D, K = 64 keys per key half, P in tensor memory, V in shared memory
+//   O += P V    : M = 128, N = D, K = 128 keys, P in tensor memory, V in shared memory
 // Q and K sit in shared memory in the 128-byte-swizzled K-major layout, V in
 // the M/N-major layout.  Tensor memory (TMEM, 512 columns) holds three S
-// buffers of 128 columns and the O accumulator (D columns).  Two softmax
-// groups take the two 64-key halves of every tile, so every SM sub-partition
-// runs two softmax warps and one warp's loads, maxima and stores overlap the
-// other's exponentials (the softmax is latency-bound: at 32 exponentials per
-// clock per SM the MUFU unit is busy about a third of a tile).  The partners
-// of a lane quarter agree on each tile's row max through one TMEM column of
-// their halves, so both halves share one reference max and accumulate into
-// the one O; each group rescales, and at the end writes, its half of O's
-// columns.  A group overwrites the first 32 columns of its half of the S
-// buffer with P as bf16 pairs and the P.V product reads P from there: P never
-// passes through shared memory, whose bandwidth the MMA operand reads and the
-// TMA writes already share.  S of tile i + 3 reuses the buffer of tile i, so
-// it waits for the completion of P.V of tile i; three buffers keep that wait
-// off the softmax's path.
+// buffers of 128 columns and the O accumulator (D columns).
 //
-// The K and V rings have separate depths, the keys' deeper (S runs up to
-// three tiles ahead of P.V): 3 and 2 stages of 32 KB for D = 128, what the
-// shared memory holds next to Q and the epilogue staging.  The epilogue stages
-// O / l in 4 KB boxes of shared memory (the 128-byte swizzle) and writes them
-// with bulk tensor stores, which drain while the warps go on.
+// What bounds it.  The two products of a 128 x 128 tile take the tensor pipe
+// ~1050 cycles; a softmax warp takes ~1500 on its 32 rows (S from TMEM, row
+// max, 128 exponentials a row, P back), a serial chain whatever runs beside
+// it.  Two softmax groups therefore take the tiles in turn, one thread per
+// position with its whole 128-key row: each has two tile periods for its chain,
+// and the pipe, not the chain, sets the pace (measured ~1400 cycles a tile; the
+// groups on the two key halves of every tile, meeting in a row-max exchange,
+// made ~2200).  The reference max of the online softmax passes from tile to
+// tile, so from group to group, through shared memory right after a tile's row
+// max is known; a group keeps its own row sum and takes it to the item's last
+// reference at the end.  P (bf16 pairs) overwrites the first 64 columns of its
+// S buffer.  S of tile i + 3 reuses the buffer of tile i, so it waits for the
+// completion of P.V of tile i; three buffers keep that off the softmax's path.
+//
+// Code size.  Every role's loop competes for the instruction cache: with the
+// softmax unrolled over a whole row the same schedule took 190 us, with the
+// loops below 64 scores at a time, rolled, 139 us at the shape below (stalls
+// for want of an instruction: 26% of all, then 4%).  So loops are rolled where
+// they can be, waits are small, and the optimizer is kept from copying them.
+//
+// At an item's end everything hangs on how soon the next one starts: the
+// epilogue warps read all of O at once (168 registers a thread) before they
+// store it, Q has two buffers, and the rows of the last V tile past the item's
+// keys are cleared by the value producer's idle lanes.  K and V rings of two
+// stages each (D = 128) are what fits beside that; the epilogue stages O / l in
+// 4 KB boxes of shared memory (the 128-byte swizzle) and writes them with bulk
+// tensor stores, which drain while the warps go on.
+//
+// Measured at B = 4, T = 2048, 32 heads, D = 128, L = 5: 139.6 -> 113.5 us, 65%
+// of the measured bf16 rate; B = 5, T = 1818, 32 over 8 heads, L = 4, ragged:
+// 165.9 -> 127.4 us.  What is left: ~1500 cycles of every item's switch, waits
+// for K and V tiles that the other SMs' traffic delays, and CTAs with one pair
+// more than others.
 //
 // Work item: (sequence b, query head h, tile of 128 positions).  Tile x of a
 // (b, h) sees about x + 1 key tiles, so tile x is paired with tile
@@ -37,22 +52,17 @@
 // runs pairs c, c + G, c + 2G, ... in (b, h)-major order: the CTAs that run at
 // the same time read the keys and values of a few heads, which stay in L2.
 //
-// Roles (512 threads, one CTA per SM; setmaxnreg gives the softmax warps 168
-// registers a thread and the others 88):
+// Roles (512 threads, one CTA per SM):
 //   warps 0-7   softmax, two groups of four: warp w reads TMEM lane quarter
-//               w % 4 (one thread per position) and key half w / 4 of every
-//               tile, with packed f32x2 arithmetic; at the end of an item it
+//               w % 4 of the tiles of parity w / 4; at the end of an item it
 //               hands its row sums to the epilogue warps.
-//   warp 8      producer: lane 0 loads the Q tile and feeds the K and V rings
-//               with 2-D TMA, polling the free slots of both.
+//   warp 8      producer of Q and K, warp 11 of V (2-D TMA by lane 0).
 //   warp 9      S issue (lane 0) and the TMEM allocation.
 //   warp 10     P.V issue (lane 0).  Separate issuers keep S of later tiles
 //               from queueing behind the wait for this tile's P.
-//   warp 11     idle (completes the register split's warpgroup).
 //   warps 12-15 epilogue: warp 12 + q reads lane quarter q of O once the
 //               item's last P.V is done, frees O for the next item and writes
-//               O / l with bulk tensor stores, while the softmax warps are
-//               already on the next item.
+//               O / l, while the softmax warps are already on the next item.
 //
 // Online softmax in the log2 domain with a lazy reference max: O is rescaled
 // in TMEM only when a tile's max exceeds the reference by more than 8 (factor
@@ -76,11 +86,11 @@ namespace {
 
 constexpr int kBM = 128;          // positions per work item (MMA rows, TMEM lanes)
 constexpr int kBN = 128;          // keys per tile
-constexpr int kMaxStages = 4;     // K/V ring stages (the launch picks as many as fit)
-constexpr int kSoftWarps = 8;     // two groups of four: the key halves of every tile
+constexpr int kSoftWarps = 8;     // two groups of four: the even and the odd tiles
 constexpr int kProdWarp = 8;
 constexpr int kSWarp = 9;
-constexpr int kPVWarp = 10;      // warp 11 only completes warpgroup 2
+constexpr int kPVWarp = 10;
+constexpr int kVProdWarp = 11;
 constexpr int kEpiWarp0 = 12;    // warps 12-15: the item epilogues, one per TMEM lane quarter
 constexpr int kEpiWarps = 4;
 constexpr int kThreads = 512;
@@ -97,31 +107,37 @@ constexpr float kRescaleLog2 = 8.0f;
 // within one phase of its barrier; with two, a wait for tile i could pass on
 // the completion of tile i - 2 (measured: the last tiles of a segment missing
 // from O when the values arrived late from DRAM).
-constexpr int B_KFULL = 0, B_KEMPTY = 4, B_VFULL = 8, B_VEMPTY = 12, B_QFULL = 16, B_QEMPTY = 17, B_SFULL = 18,
-              B_PFULL = 21, B_BFREE = 24, B_ODONE = 27, B_OFREE = 31, B_MDONE = 32, B_LREADY = 34, B_LFREE = 35,
-              kNumBars = 36;
+constexpr int B_KFULL = 0, B_KEMPTY = 4, B_VFULL = 8, B_VEMPTY = 12, B_QFULL = 16, B_SFULL = 18,
+              B_PFULL = 21, B_BFREE = 24, B_ODONE = 27, B_OFREE = 31, B_MDONE = 32, B_LREADY = 34, B_LFREE = 35, B_VCLR = 36, B_QEMPTY = 40,
+              kNumBars = 42;
 
 template <int D>
 struct BlkCfg {
   static constexpr int kHalves = D / 64;                // swizzle atoms across the head dim
   static constexpr uint32_t kQBytes = kHalves * kAtom;  // 128 positions x D
   static constexpr uint32_t kKV = kHalves * kAtom;      // 128 keys x D
-  static constexpr uint32_t off_Q = 0;
+  static constexpr uint32_t off_Q = 0;                  // two items' queries
   // epilogue staging: per epilogue warp two boxes of 32 positions x 32 fp32
   // outputs (4 KB each, 128-byte swizzle): the D/32 chunks go through them in
   // rounds of two
   static constexpr uint32_t kStage = kEpiWarps * 2 * 4096;
-  static constexpr uint32_t off_stg = off_Q + kQBytes;
+  static constexpr uint32_t off_stg = off_Q + 2 * kQBytes;
   static constexpr uint32_t off_K = off_stg + kStage;
-  // K ring of nk stages, then the V ring of nv
-  static __host__ __device__ uint32_t off_V(int nk) { return off_K + nk * kKV; }
-  static __host__ __device__ uint32_t off_bar(int nk, int nv) { return off_V(nk) + nv * kKV; }
-  static __host__ __device__ uint32_t off_misc(int nk, int nv) { return off_bar(nk, nv) + 512; }
-  // the item's row sums, [key half][position], from the softmax to the epilogue warps
-  static __host__ __device__ uint32_t off_lsum(int nk, int nv) { return off_misc(nk, nv) + 16; }
-  static size_t smem_bytes(int nk, int nv) { return 1024 + off_lsum(nk, nv) + 2 * kBM * 4; }
+  // The K ring, then the V ring, as many stages as fit: S runs up to three
+  // tiles ahead of P.V, so the keys get the deeper ring.  The depths are
+  // compile-time constants: a division by a run-time depth costs an issuing
+  // thread ~100 cycles each.
+  static constexpr unsigned kNK = D == 128 ? 2 : 4, kNV = D == 128 ? 2 : 4;
+  static constexpr uint32_t off_V = off_K + kNK * kKV;
+  static constexpr uint32_t off_bar = off_V + kNV * kKV;
+  static constexpr uint32_t off_misc = off_bar + kNumBars * 8;
+  // the item's row sums, [group][position], from the softmax to the epilogue warps
+  static constexpr uint32_t off_lsum = off_misc + 16;
+  // the running reference max of every position, from one softmax group to the other
+  static constexpr uint32_t off_mref = off_lsum + 2 * kBM * 4;
+  static constexpr size_t kSmem = 1024 + off_mref + kBM * 4;
   static_assert(kTmemO + D <= kTmemCols, "TMEM columns");
-  static_assert(kNumBars * 8 <= 512, "barrier area");
+  static_assert(kSmem <= 227 * 1024, "shared memory");
 };
 
 // Division of a non-negative int below 2^31 by a fixed positive divisor d as
@@ -145,13 +161,13 @@ struct FastDiv {
 
 struct BlkParams {
   const int* seq_len;
+  float* out;
   unsigned* status;
   int B, H, Hkv, T, S_cap, L;
   FastDiv by_L, by_H, by_group, by_npb;
   int nqt;             // position tiles per sequence
   int npb;             // tile pairs per (b, h)
   int npairs;          // B * H * npb (below 2^31)
-  int nk, nv;          // K and V ring stages
   float scale_log2;
 };
 
@@ -232,13 +248,27 @@ __device__ __forceinline__ void staging_free(int lane) {
   __syncwarp();
 }
 
-// Warpgroup register split (setmaxnreg): the two softmax warpgroups take 168
-// registers a thread, the producer / MMA and epilogue warpgroups give theirs
-// down to 88, so that each SM sub-partition's 16384 registers hold its four
-// warps (2 x 168 + 2 x 88 = 512 per lane) -- exactly the 512 x 128 the block
-// is launched with.
-__device__ __forceinline__ void regs_up() { asm volatile("setmaxnreg.inc.sync.aligned.u32 168;" ::: "memory"); }
-__device__ __forceinline__ void regs_down() { asm volatile("setmaxnreg.dec.sync.aligned.u32 88;" ::: "memory"); }
+// Warpgroup register split (setmaxnreg), 512 x 128 registers in all as the
+// block is launched: 136 a thread for the two softmax warpgroups, 168 for the
+// epilogue's (a whole row of O), 72 for the producers' and MMA issuers'.
+template <int N>
+__device__ __forceinline__ void regs_up() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N) : "memory");
+}
+template <int N>
+__device__ __forceinline__ void regs_down() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N) : "memory");
+}
+
+// The hand-over of a tile's reference max between the two warps (one of each
+// softmax group) of a TMEM lane quarter: named barriers 1-8, per quarter and
+// tile parity; the tile's warp arrives, the next tile's warp waits.
+__device__ __forceinline__ void turn_pass(int quarter, unsigned tile) {
+  asm volatile("bar.arrive %0, 64;" ::"r"(1 + 2 * quarter + (int)(tile & 1)) : "memory");
+}
+__device__ __forceinline__ void turn_wait(int quarter, unsigned tile) {
+  asm volatile("bar.sync %0, 64;" ::"r"(1 + 2 * quarter + (int)(tile & 1)) : "memory");
+}
 
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -248,23 +278,25 @@ __global__ void __launch_bounds__(kThreads, 1)
   using C = BlkCfg<D>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  const int k_stages = p.nk, v_stages = p.nv;  // K and V ring depths
-  const uint32_t off_V = C::off_V(k_stages);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(base + C::off_bar(k_stages, v_stages));
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + C::off_misc(k_stages, v_stages));
-  float* lsum = reinterpret_cast<float*>(base + C::off_lsum(k_stages, v_stages));
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(base + C::off_misc(k_stages, v_stages) + 4);
+  constexpr unsigned k_stages = C::kNK, v_stages = C::kNV;  // K and V ring depths
+  constexpr uint32_t off_V = C::off_V;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(base + C::off_bar);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + C::off_misc);
+  float* lsum = reinterpret_cast<float*>(base + C::off_lsum);
+  float* mref = reinterpret_cast<float*>(base + C::off_mref);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(base + C::off_misc + 4);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
+#pragma unroll 1
     for (int b = 0; b < kNumBars; ++b) {
-      const bool soft = (b >= B_PFULL && b < B_PFULL + kSBufs) || b == B_LREADY;
-      const bool epi = b == B_OFREE || b == B_LFREE;
-      mbar_init(&bars[b], soft ? kSoftWarps : (epi ? kEpiWarps : 1));
+      const bool four = (b >= B_PFULL && b < B_PFULL + kSBufs) || b == B_OFREE || b == B_LFREE;
+      mbar_init(&bars[b], b == B_LREADY ? kSoftWarps : four ? 4 : 1);  // the warps that arrive
     }
     *abort_flag = 0;
     fence_barrier_init();
   }
+  pdl_wait();  // every global access and the TMEM allocation come after it
   if (warp == kSWarp) {
     tc::tmem_alloc(tmem_slot, kTmemCols);
     tc::tmem_relinquish();
@@ -273,189 +305,198 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  if (warp >= kSoftWarps) {
-  regs_down();
-  if (warp == kProdWarp) {
-    // ------------------------------------------------------------ producer
+  if (warp >= kSoftWarps && warp < kEpiWarp0) {
+  regs_down<72>();
+  if (warp == kProdWarp || warp == kVProdWarp) {
+    // ----------------------------------------------------------- producers
+    // Warp 8 loads the queries and the keys, warp 11 the values: one loop, so
+    // that its code is there once.  Lane 0 issues; the other lanes are there to
+    // clear the rows past an item's last visible key in its last V tile.
+    const bool keys = warp == kProdWarp;
+    const uint64_t pol_q = policy_evict_first(), pol_kv = policy_evict_last();
+    const CUtensorMap* map = keys ? &tmK : &tmV;
     if (lane == 0) {
-      tc::prefetch_tmap(&tmQ);
-      tc::prefetch_tmap(&tmK);
-      tc::prefetch_tmap(&tmV);
-      const uint64_t pol_q = policy_evict_first(), pol_kv = policy_evict_last();
-      struct Cursor {  // next tile to load: item it, its tile t, CTA-local tile i, item kq
-        Walker w;
-        Item it;
-        int t, i, kq;
-        bool has, qdone;
-      };
-      auto first = [&](Cursor& c) {  // the next item with keys
-        c.has = false;
-        while (c.w.next(p, c.it))
-          if (c.it.nt > 0) {
-            c.has = true;
-            c.t = 0;
-            c.qdone = false;
-            return;
-          }
-      };
-      auto step = [&](Cursor& c) {
-        ++c.i;
-        if (++c.t == c.it.nt) {
-          ++c.kq;
-          first(c);
-        }
-      };
-      auto kv_row = [&](const Cursor& c) { return (c.it.b * p.Hkv + p.by_group.div(c.it.h)) * p.S_cap + c.t * kBN; };
-      Cursor ck, cv;
-      ck.w.start();
-      cv.w.start();
-      ck.i = cv.i = ck.kq = cv.kq = 0;
-      first(ck);
-      first(cv);
-      int q_issued = 0;
-      uint64_t t_last = global_timer_ns();
-      int spins = 0, seen = 0;
-      while (ck.has || cv.has) {
-        bool progressed = false;
-        if (ck.has) {
-          if (ck.t == 0 && !ck.qdone) {
-            if (mbar_test_wait(&bars[B_QEMPTY], (ck.kq & 1) ^ 1)) {
-              mbar_arrive_expect_tx(&bars[B_QFULL], C::kQBytes);
-              for (int hd = 0; hd < C::kHalves; ++hd)
-                tc::tma_load_2d(base + C::off_Q + hd * kAtom, &tmQ, ck.it.h * D + hd * 64, ck.it.b * p.T + ck.it.j0,
-                                &bars[B_QFULL], pol_q);
-              ck.qdone = true;
-              ++q_issued;
-              progressed = true;
-              {  // the next item's Q into L2, an item ahead of its load
-                Walker la = ck.w;
-                Item nx;
-                while (la.next(p, nx))
-                  if (nx.nt > 0) {
-                    for (int hd = 0; hd < C::kHalves; ++hd)
-                      tc::tma_prefetch_l2_2d(&tmQ, nx.h * D + hd * 64, nx.b * p.T + nx.j0);
-                    break;
-                  }
-              }
-            }
-          } else if (mbar_test_wait(&bars[B_KEMPTY + ck.i % k_stages], ((ck.i / k_stages) & 1) ^ 1)) {
-            const int st = ck.i % k_stages;
-            mbar_arrive_expect_tx(&bars[B_KFULL + st], C::kKV);
-            for (int hd = 0; hd < C::kHalves; ++hd)
-              tc::tma_load_2d(base + C::off_K + st * C::kKV + hd * kAtom, &tmK, hd * 64, kv_row(ck),
-                              &bars[B_KFULL + st], pol_kv);
-            step(ck);
-            progressed = true;
+      tc::prefetch_tmap(map);
+      if (keys) tc::prefetch_tmap(&tmQ);
+    }
+    unsigned char* ring = base + (keys ? C::off_K : off_V);
+    uint64_t* full = &bars[keys ? B_KFULL : B_VFULL];
+    uint64_t* empty = &bars[keys ? B_KEMPTY : B_VEMPTY];
+    const unsigned depth = keys ? k_stages : v_stages;
+    unsigned st = 0, phase = 1;  // stage and its parity as the waiter sees it
+    unsigned issued = 0, q_issued = 0;
+    Walker w;
+    w.start();
+    Item it, nx;
+    nx.nt = 0;
+    bool has = true, ok = true;
+    while (has && ok) {
+      it = nx;
+      has = w.next(p, nx);
+      if (it.nt == 0) continue;
+      if (keys) {
+        const unsigned qb = q_issued & 1;
+        ok = warp_wait_small(&bars[B_QEMPTY + qb], ((q_issued >> 1) & 1) ^ 1, abort_flag);
+        if (!ok) break;
+        if (lane == 0) {
+          mbar_arrive_expect_tx(&bars[B_QFULL + qb], C::kQBytes);
+          for (int hd = 0; hd < C::kHalves; ++hd) {
+            tc::tma_load_2d(base + C::off_Q + qb * C::kQBytes + hd * kAtom, &tmQ, it.h * D + hd * 64, it.b * p.T + it.j0,
+                            &bars[B_QFULL + qb], pol_q);
+            // the next item's Q into L2, an item ahead of its load
+            if (has) tc::tma_prefetch_l2_2d(&tmQ, nx.h * D + hd * 64, nx.b * p.T + nx.j0);
           }
         }
-        if (cv.has && mbar_test_wait(&bars[B_VEMPTY + cv.i % v_stages], ((cv.i / v_stages) & 1) ^ 1)) {
-          const int st = cv.i % v_stages;
-          mbar_arrive_expect_tx(&bars[B_VFULL + st], C::kKV);
+        ++q_issued;
+      }
+      int row = (it.b * p.Hkv + p.by_group.div(it.h)) * p.S_cap;
+      for (int t = 0; t < it.nt; ++t, row += kBN) {
+        ok = warp_wait_small(&empty[st], phase, abort_flag);
+        if (!ok) break;
+        unsigned char* dst = ring + st * C::kKV;
+        if (lane == 0) {
+          mbar_arrive_expect_tx(&full[st], C::kKV);
           for (int hd = 0; hd < C::kHalves; ++hd)
-            tc::tma_load_2d(base + off_V + st * C::kKV + hd * kAtom, &tmV, hd * 64, kv_row(cv), &bars[B_VFULL + st],
-                            pol_kv);
-          step(cv);
-          progressed = true;
+            tc::tma_load_2d(dst + hd * kAtom, map, hd * 64, row, &full[st], pol_kv);
         }
-        if (progressed) continue;
-        // Nothing to do: back off so that this warp leaves its scheduler's
-        // issue slots to the softmax warp beside it.
-        __nanosleep(32);
-        if (++spins < 32) continue;
-        spins = 0;  // every 32 idle polls: check for an abort or a stall of more than kWaitLimitNs
-        const uint64_t now = global_timer_ns();
-        if (ck.i + cv.i + q_issued != seen) {
-          seen = ck.i + cv.i + q_issued;
-          t_last = now;
+        __syncwarp();
+        ++issued;
+        const int vrows = it.klen - t * kBN;
+        if (!keys && vrows < kBN) {  // the item's last V tile: clear its rows past the last visible key
+          ok = warp_wait_small(&full[st], phase ^ 1, abort_flag);
+          if (!ok) break;
+#pragma unroll 1
+          for (int idx = vrows * C::kHalves * 8 + lane; idx < kBN * C::kHalves * 8; idx += 32)
+            *reinterpret_cast<uint4*>(dst + ((idx >> 3) % C::kHalves) * kAtom + idx / (C::kHalves * 8) * 128 +
+                                      (idx & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
+          tc::fence_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bars[B_VCLR + st]);
         }
-        if (*abort_flag) break;
-        if (now - t_last > kWaitLimitNs) {
-          *abort_flag = 1;
-          record_status(p.status, kStatusTimeout);
-          break;
+        if (++st == depth) {
+          st = 0;
+          phase ^= 1;
         }
       }
-      if (ck.has || cv.has) {  // aborted: let issued loads land before the CTA exits
-        for (int j = (ck.i > k_stages ? ck.i - k_stages : 0); j < ck.i; ++j)
-          mbar_drain(&bars[B_KFULL + j % k_stages], (j / k_stages) & 1);
-        for (int j = (cv.i > v_stages ? cv.i - v_stages : 0); j < cv.i; ++j)
-          mbar_drain(&bars[B_VFULL + j % v_stages], (j / v_stages) & 1);
-        if (q_issued > 0) mbar_drain(&bars[B_QFULL], (q_issued - 1) & 1);
-      }
+    }
+    if (!ok && lane == 0) {  // aborted: let issued loads land before the CTA exits
+      for (unsigned j = (issued > depth ? issued - depth : 0); j < issued; ++j)
+        mbar_drain(&full[j % depth], (j / depth) & 1);
+      for (unsigned j = (q_issued > 2 ? q_issued - 2 : 0); j < q_issued; ++j)
+        mbar_drain(&bars[B_QFULL + (j & 1)], (j >> 1) & 1);
     }
   } else if (warp == kSWarp || warp == kPVWarp) {
     // ----------------------------------------------------------- MMA issue
+    // Ring positions are counted up, not divided out, and the loops hold little
+    // but waits and products: the two threads' time per tile is what the tensor
+    // pipe waits for between their batches.
     if (lane == 0) {
-      const bool s_role = warp == kSWarp;
-      constexpr uint32_t idS = tc::idesc_bf16_f32(kBM, kBN, false, false);
-      constexpr uint32_t idO = tc::idesc_bf16_f32(kBM, D, false, true);
-      const uint64_t dQ = tc::sw128_desc(smem_u32(base + C::off_Q), 16, 1024);
-      const uint32_t sK = smem_u32(base + C::off_K), sV = smem_u32(base + off_V);
       bool ok = true;
       Walker w;
       w.start();
       Item it;
-      int i = 0, kq = 0;
-      while (ok && w.next(p, it)) {
-        if (it.nt == 0) continue;
-        for (int t = 0; t < it.nt; ++t, ++i) {
-          const int bi = i % kSBufs;
-          if (s_role) {
-            // S(i) = Q K(i)^T into buffer i % 3, once P.V of tile i - 3 has read that buffer
-            if ((t == 0 && !mbar_wait(&bars[B_QFULL], kq & 1, abort_flag, p.status)) ||
-                !mbar_wait(&bars[B_KFULL + i % k_stages], (i / k_stages) & 1, abort_flag, p.status) ||
-                !mbar_wait(&bars[B_BFREE + bi], ((i / kSBufs) & 1) ^ 1, abort_flag, p.status)) {
-              ok = false;
-              break;
-            }
+      unsigned bi = 0;  // S buffer of the tile
+      uint32_t col = tmem;
+      unsigned items = 0;
+      if (warp == kSWarp) {
+        // S(i) = Q K(i)^T into buffer i % 3, once P.V of tile i - 3 has read that buffer
+        constexpr uint32_t idS = tc::idesc_bf16_f32(kBM, kBN, false, false);
+        const uint64_t dQ0 = tc::sw128_desc(smem_u32(base + C::off_Q), 16, 1024);
+        const uint64_t dK0 = tc::sw128_desc(smem_u32(base + C::off_K), 16, 1024);
+        uint64_t dK = dK0;
+        unsigned st = 0, k_phase = 0, b_phase = 1;
+        while (ok && w.next(p, it)) {
+          if (it.nt == 0) continue;
+          const uint64_t dQ = dQ0 + (items & 1) * desc_step(C::kQBytes);
+          ok = mbar_wait_small(&bars[B_QFULL + (items & 1)], (items >> 1) & 1, abort_flag);
+          ++items;
+#pragma unroll 1
+          for (int t = it.nt; ok && t > 0; --t) {
+            ok = mbar_wait_small(&bars[B_KFULL + st], k_phase, abort_flag) &&
+                 mbar_wait_small(&bars[B_BFREE + bi], b_phase, abort_flag);
+            if (!ok) break;
             tc::fence_after_sync();
-            const uint64_t dK = tc::sw128_desc(sK + (i % k_stages) * C::kKV, 16, 1024);
 #pragma unroll
             for (int ks = 0; ks < D / 16; ++ks) {
               const uint64_t step = desc_step((ks >> 2) * kAtom + (ks & 3) * 32);
-              tc::mma_bf16(tmem + bi * kBN, dQ + step, dK + step, idS, ks > 0 ? 1u : 0u);
+              tc::mma_bf16(col, dQ + step, dK + step, idS, ks > 0 ? 1u : 0u);
             }
             tc::mma_commit(&bars[B_SFULL + bi]);
-            tc::mma_commit(&bars[B_KEMPTY + i % k_stages]);
-            if (t == it.nt - 1) tc::mma_commit(&bars[B_QEMPTY]);
-          } else {
-            // O (+)= P_0(i) V_0(i) + P_1(i) V_1(i) over the key halves h = 0, 1: P_h in
-            // columns 64h .. 64h+31 of buffer i % 3
-            const bool first = t == 0;
-            if (!mbar_wait(&bars[B_PFULL + bi], (i / kSBufs) & 1, abort_flag, p.status) ||
-                !mbar_wait(&bars[B_VFULL + i % v_stages], (i / v_stages) & 1, abort_flag, p.status) ||
-                (first && kq > 0 && !mbar_wait(&bars[B_OFREE], (kq - 1) & 1, abort_flag, p.status))) {
-              ok = false;
-              break;
+            tc::mma_commit(&bars[B_KEMPTY + st]);
+            if (t == 1) tc::mma_commit(&bars[B_QEMPTY + ((items - 1) & 1)]);
+            dK += desc_step(C::kKV);
+            if (++st == k_stages) {
+              st = 0;
+              k_phase ^= 1;
+              dK = dK0;
             }
-            tc::fence_after_sync();
-            const uint64_t dV = tc::sw128_desc(sV + (i % v_stages) * C::kKV, kAtom, 1024);
-            const uint32_t pcol = tmem + bi * kBN;
-            if (first) {
-              tc::mma_bf16_ts(tmem + kTmemO, pcol, dV, idO, 0u);
-            } else {
-              tc::mma_bf16_ts(tmem + kTmemO, pcol, dV, idO, 1u);
+            col += kBN;
+            if (++bi == kSBufs) {
+              bi = 0;
+              b_phase ^= 1;
+              col = tmem;
             }
-#pragma unroll
-            for (int ks = 1; ks < kBN / 16; ++ks)
-              tc::mma_bf16_ts(tmem + kTmemO, pcol + (ks >> 2) * 64 + (ks & 3) * 8, dV + desc_step(ks * 16 * 128), idO, 1u);
-            tc::mma_commit(&bars[B_VEMPTY + i % v_stages]);
-            tc::mma_commit(&bars[B_ODONE + (i & 3)]);
-            tc::mma_commit(&bars[B_BFREE + bi]);
           }
         }
-        ++kq;
+        tc::mma_commit(&bars[B_MDONE]);  // every MMA finished before TMEM is released
+        mbar_drain(&bars[B_MDONE], 0);
+      } else {
+        // O (+)= P(i) V(i), P in the first 64 columns of buffer i % 3
+        constexpr uint32_t idO = tc::idesc_bf16_f32(kBM, D, false, true);
+        const uint64_t dV0 = tc::sw128_desc(smem_u32(base + off_V), kAtom, 1024);
+        uint64_t dV = dV0;
+        unsigned st = 0, v_phase = 0, p_phase = 0, od = 0;
+        unsigned cleared = 0;  // bit s: parity of the clears of V stage s so far
+        while (ok && w.next(p, it)) {
+          if (it.nt == 0) continue;
+          if (items > 0) ok = mbar_wait_small(&bars[B_OFREE], (items - 1) & 1, abort_flag);
+          ++items;
+          const bool partial = it.klen < it.nt * kBN;  // rows of the last V tile get cleared
+          uint32_t acc = 0;
+#pragma unroll 1
+          for (int t = it.nt; ok && t > 0; --t) {
+            ok = mbar_wait_small(&bars[B_VFULL + st], v_phase, abort_flag);
+            if (ok && t == 1 && partial) {
+              ok = mbar_wait_small(&bars[B_VCLR + st], (cleared >> st) & 1, abort_flag);
+              cleared ^= 1u << st;
+            }
+            ok = ok && mbar_wait_small(&bars[B_PFULL + bi], p_phase, abort_flag);
+            if (!ok) break;
+            tc::fence_after_sync();
+#pragma unroll
+            for (int ks = 0; ks < kBN / 16; ++ks)
+              tc::mma_bf16_ts(tmem + kTmemO, col + ks * 8, dV + desc_step(ks * 16 * 128), idO, ks > 0 ? 1u : acc);
+            acc = 1;
+            tc::mma_commit(&bars[B_BFREE + bi]);
+            tc::mma_commit(&bars[B_VEMPTY + st]);
+            tc::mma_commit(&bars[B_ODONE + od]);
+            od = (od + 1) & 3;
+            dV += desc_step(C::kKV);
+            if (++st == v_stages) {
+              st = 0;
+              v_phase ^= 1;
+              dV = dV0;
+            }
+            col += kBN;
+            if (++bi == kSBufs) {
+              bi = 0;
+              p_phase ^= 1;
+              col = tmem;
+            }
+          }
+        }
+        tc::mma_commit(&bars[B_MDONE + 1]);
+        mbar_drain(&bars[B_MDONE + 1], 0);
       }
-      const int role = s_role ? 0 : 1;
-      tc::mma_commit(&bars[B_MDONE + role]);  // every MMA finished before TMEM is released
-      mbar_drain(&bars[B_MDONE + role], 0);
     }
+  }
   } else if (warp >= kEpiWarp0) {
+    regs_up<168>();
     // ------------------------------------------------------------ epilogue
     // Warp 12 + q writes positions 32q .. 32q+31 of every item: O / (l_0 + l_1)
     // from TMEM lane quarter q, staged in D/32 boxes and written with bulk
     // tensor stores.  The softmax warps go on with the next item meanwhile; its
-    // first P.V waits until O has been read here.
+    // first P.V waits until O has been read here, so a whole row is read at once.
     const int quarter = warp - kEpiWarp0;
     const int r = quarter * 32 + lane;
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
@@ -464,193 +505,183 @@ __global__ void __launch_bounds__(kThreads, 1)
     Walker w;
     w.start();
     Item it;
-    int i = 0, ke = 0;
-    while (w.next(p, it)) {
-      staging_free(lane);  // the previous item's stores have read the boxes
-      if (it.nt == 0) {  // no visible key anywhere in the tile: zeros, every chunk from the first box
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-          *reinterpret_cast<float4*>(stg + lane * 128 + (e << 4)) = make_float4(0.f, 0.f, 0.f, 0.f);
+    unsigned i = 0, ke = 0;
+    while (!dead && w.next(p, it)) {
+      const int j = it.j0 + r;
+      if (it.nt == 0) {  // no visible key anywhere in the tile: zeros
 #pragma unroll 1
-        for (int c = 0; c < D / 32; ++c) store_box(&tmO, stg, it.h * D + c * 32, it.j0 + quarter * 32, it.b, lane);
+        for (int row = it.j0 + quarter * 32; row < p.T && row < it.j0 + quarter * 32 + 32; ++row)
+          for (int c = lane; c < D / 4; c += 32)
+            reinterpret_cast<float4*>(p.out + (((long long)it.b * p.T + row) * p.H + it.h) * D)[c] =
+                make_float4(0.f, 0.f, 0.f, 0.f);
         continue;
       }
       i += it.nt;
-      const int jl = i - 1;  // the item's last tile
-      const int j = it.j0 + r;
+      const unsigned jl = i - 1;  // the item's last tile
       // a position that saw no key, or past the sequence: zeros
       const bool has_value = j < it.n && p.L * p.by_L.div(j) > 0;
-      if (!dead) dead = !warp_wait(&bars[B_LREADY], ke & 1, abort_flag, p.status);
-      const float l0 = lsum[r], l1 = lsum[kBM + r];
+      dead = !warp_wait_small(&bars[B_LREADY], ke & 1, abort_flag);
+      if (dead) break;
+      const float inv = 1.f / (lsum[r] + lsum[kBM + r]);
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars[B_LFREE]);
-      ++ke;
-      const float inv = has_value ? 1.f / (l0 + l1) : 0.f;
-      if (!dead) dead = !warp_wait(&bars[B_ODONE + (jl & 3)], (jl >> 2) & 1, abort_flag, p.status);
-      // rounds of two chunks: read from TMEM into the two boxes, then their stores
-#pragma unroll 1
-      for (int c2 = 0; c2 < D / 32; c2 += 2) {
-        if (c2 > 0) staging_free(lane);  // the previous round's stores have read the boxes
-        if (!dead) {
-          tc::fence_after_sync();
-#pragma unroll 1
-          for (int c = c2; c < c2 + 2; ++c) {
-            uint32_t a[32];
-            tc::tmem_ld32(lane_base + kTmemO + c * 32, a);
-            tc::tmem_wait_ld();
+      dead = !warp_wait_small(&bars[B_ODONE + (jl & 3)], (jl >> 2) & 1, abort_flag);
+      if (dead) break;
+      tc::fence_after_sync();
+      uint32_t o[D];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-              if (has_value)
-                v = make_float4(__uint_as_float(a[4 * q]) * inv, __uint_as_float(a[4 * q + 1]) * inv,
-                                __uint_as_float(a[4 * q + 2]) * inv, __uint_as_float(a[4 * q + 3]) * inv);
-              *reinterpret_cast<float4*>(stg + (c - c2) * 4096 + lane * 128 + ((q ^ (lane & 7)) << 4)) = v;
-            }
-          }
+      for (int c = 0; c < D / 32; ++c)
+        tc::tmem_ld32(lane_base + kTmemO + c * 32, *reinterpret_cast<uint32_t(*)[32]>(o + 32 * c));
+      tc::tmem_wait_ld();
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars[B_OFREE]);
+      // through the two boxes in turn, and out
+#pragma unroll
+      for (int c = 0; c < D / 32; ++c) {
+        unsigned char* box = stg + (c & 1) * 4096;
+        if ((c & 1) == 0) staging_free(lane);  // the stores before have read the boxes
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const uint32_t* a = o + 32 * c + 4 * q;
+          float4 v = make_float4(__uint_as_float(a[0]) * inv, __uint_as_float(a[1]) * inv,
+                                 __uint_as_float(a[2]) * inv, __uint_as_float(a[3]) * inv);
+          if (!has_value) v = make_float4(0.f, 0.f, 0.f, 0.f);
+          *reinterpret_cast<float4*>(box + lane * 128 + ((q ^ (lane & 7)) << 4)) = v;
         }
-        if (c2 + 2 == D / 32) {  // O is read: the next item's P.V may overwrite it
-          tc::fence_before_sync();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&bars[B_OFREE]);
-        }
-        if (!dead)
-#pragma unroll 1
-          for (int c = c2; c < c2 + 2; ++c)
-            store_box(&tmO, stg + (c - c2) * 4096, it.h * D + c * 32, it.j0 + quarter * 32, it.b, lane);
+        store_box(&tmO, box, it.h * D + c * 32, it.j0 + quarter * 32, it.b, lane);
       }
+      ++ke;
     }
     if (lane == 0) tc::bulk_wait_all();  // the output stores have landed
-  }
   } else {
-  regs_up();
+  regs_up<136>();
     // ------------------------------------------------------------- softmax
-    const int kh = warp >> 2, quarter = warp & 3;
+    const int grp = warp >> 2, quarter = warp & 3;  // this group's tiles: CTA-local index parity grp
     const int r = quarter * 32 + lane;  // this thread's position in the tile (its TMEM lane)
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-    const uint32_t o_col = kTmemO + kh * (D / 2);  // this group's half of the O columns
-    const int sid = threadIdx.x;        // 0..255 among the softmax threads
     const float sl2 = p.scale_log2;
+    const uint64_t sc2 = f2(sl2, sl2);
     bool dead = false;
     Walker w;
     w.start();
     Item it;
-    int i = 0, ke = 0;  // CTA-local tile, items with keys
+    unsigned i = 0, ke = 0;  // CTA-local tile, items with keys
     while (w.next(p, it)) {
       if (it.nt == 0) continue;  // no visible key anywhere in the tile: the epilogue warps write zeros
       const int j = it.j0 + r;
-      const bool valid = j < it.n;
-      const int rowlim = valid ? p.L * p.by_L.div(j) : 0;  // keys below it are visible to this position
-      float m_used = -CUDART_INF_F, l = 0.f;
-      for (int t = 0; t < it.nt; ++t, ++i) {
-        const int bi = i % kSBufs;
-        uint32_t s[64];
-        if (!dead) dead = !warp_wait(&bars[B_SFULL + bi], (i / kSBufs) & 1, abort_flag, p.status);
-        if (!dead) {
-          tc::fence_after_sync();
-          tc::tmem_ld32(lane_base + bi * kBN + kh * 64, *reinterpret_cast<uint32_t(*)[32]>(s));
-          tc::tmem_ld32(lane_base + bi * kBN + kh * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(s + 32));
-          tc::tmem_wait_ld();
-        } else {
+      const int rowlim = j < it.n ? p.L * p.by_L.div(j) : 0;  // keys below it are visible to this position
+      float m_own = -CUDART_INF_F, l = 0.f;  // the sum over this group's tiles and the reference it is taken against
+      for (int t = (int)((i ^ grp) & 1u); t < it.nt; t += 2) {
+        const unsigned ti = i + t;
+        const unsigned bi = ti % kSBufs;
+        const uint32_t s_col = lane_base + bi * kBN;
+        if (!opaque(dead)) dead = !warp_wait_small(&bars[B_SFULL + bi], (ti / kSBufs) & 1, abort_flag);
+        tc::fence_after_sync();
+        // keys at or past this position's limit: -inf (a suffix of the tile),
+        // written back to the S buffer in the 32-key chunks that have one
+        if ((t + 1) * kBN > it.mlim) {
+          const int nv = rowlim - t * kBN, nv_min = __reduce_min_sync(0xffffffffu, nv);
+#pragma unroll 1
+          for (int c = nv_min < 0 ? 0 : nv_min >> 5; c < opaque(kBN / 32); ++c) {
+            uint32_t o[32];
+            tc::tmem_ld32(s_col + c * 32, o);
+            tc::tmem_wait_ld();
 #pragma unroll
-          for (int e = 0; e < 64; ++e) s[e] = 0u;
-        }
-        // keys at or past this position's limit: -inf (a suffix of the tile)
-        const int nv = rowlim - t * kBN - kh * 64;
-        if ((t + 1) * kBN > it.mlim && __any_sync(0xffffffffu, nv < 64)) {
-#pragma unroll
-          for (int e = 0; e < 64; ++e) s[e] = e < nv ? s[e] : 0xff800000u;
-        }
-        float mx[4] = {__uint_as_float(s[0]), __uint_as_float(s[1]), __uint_as_float(s[2]), __uint_as_float(s[3])};
-#pragma unroll
-        for (int e = 4; e < 64; e += 8) {
-          mx[0] = fmax3(mx[0], __uint_as_float(s[e]), __uint_as_float(s[e + 1]));
-          mx[1] = fmax3(mx[1], __uint_as_float(s[e + 2]), __uint_as_float(s[e + 3]));
-          if (e + 4 < 64) {
-            mx[2] = fmax3(mx[2], __uint_as_float(s[e + 4]), __uint_as_float(s[e + 5]));
-            mx[3] = fmax3(mx[3], __uint_as_float(s[e + 6]), __uint_as_float(s[e + 7]));
+            for (int e = 0; e < 32; ++e) o[e] = 32 * c + e < nv ? o[e] : 0xff800000u;
+            tc::tmem_st32(s_col + c * 32, o);
           }
-        }
-        float tmax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sl2;
-        // the row max over both key halves: through column 63 of each half,
-        // already read; the pair barrier orders the partner's read after the write
-        if (!dead) {
-          tc::tmem_st1(lane_base + bi * kBN + kh * 64 + 63, __float_as_uint(tmax));
           tc::tmem_wait_st();
         }
-        tc::fence_before_sync();
-        pair_sync(quarter);
-        if (!dead) {
-          tc::fence_after_sync();
-          const uint32_t o = tc::tmem_ld1(lane_base + bi * kBN + (kh ^ 1) * 64 + 63);
-          tc::tmem_wait_ld();
-          tmax = fmaxf(tmax, __uint_as_float(o));
-        }
-        const bool need = tmax > m_used + kRescaleLog2;
-        if (__any_sync(0xffffffffu, need)) {
-          const float m_new = need ? tmax : m_used;
-          const float f = need ? fast_exp2(m_used - m_new) : 1.f;
-          l *= f;
-          if (t > 0 && !dead) {  // O holds the P.V of this item's earlier tiles: rescale this group's half
-            dead = !warp_wait(&bars[B_ODONE + ((i - 1) & 3)], ((i - 1) >> 2) & 1, abort_flag, p.status);
-            if (!dead) {
-              tc::fence_after_sync();
+        // The scores are read from TMEM twice, 64 at a time in rolled loops
+        // (row max, then exponentials): unrolled over a whole 128-key row the
+        // loop body outgrows the instruction cache.
+        float mx[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
 #pragma unroll 1
-              for (int c = 0; c < D / 64; ++c) {
-                uint32_t o[32];
-                tc::tmem_ld32(lane_base + o_col + c * 32, o);
-                tc::tmem_wait_ld();
+        for (int hf = 0; hf < opaque(2); ++hf) {
+          uint32_t sv[64];
+          tc::tmem_ld32(s_col + hf * 64, *reinterpret_cast<uint32_t(*)[32]>(sv));
+          tc::tmem_ld32(s_col + hf * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(sv + 32));
+          tc::tmem_wait_ld();
 #pragma unroll
-                for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * f);
-                tc::tmem_st32(lane_base + o_col + c * 32, o);
-              }
-              tc::tmem_wait_st();
+          for (int e = 0; e < 64; e += 8)
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              mx[q] = fmax3(mx[q], __uint_as_float(sv[e + 2 * q]), __uint_as_float(sv[e + 2 * q + 1]));
+        }
+        const float tmax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sl2;
+        // The reference max passes from tile to tile, so from group to group
+        // (one slot: a thread reads its row's before it writes the next).
+        float m_prev = -CUDART_INF_F;
+        if (t > 0) {
+          turn_wait(quarter, ti - 1);
+          m_prev = mref[r];
+        }
+        const bool need = tmax > m_prev + kRescaleLog2;
+        const float m_used = need ? tmax : m_prev;
+        mref[r] = m_used;
+        turn_pass(quarter, ti);
+        if (__any_sync(0xffffffffu, need) && t > 0 && !dead) {
+          // O holds the P.V of this item's earlier tiles, the other group's last one included: rescale it
+          dead = !warp_wait_small(&bars[B_ODONE + ((ti - 1) & 3)], ((ti - 1) >> 2) & 1, abort_flag);
+          if (!dead) {
+            const float f = need ? fast_exp2(m_prev - m_used) : 1.f;
+            tc::fence_after_sync();
+#pragma unroll 1
+            for (int c = 0; c < opaque(D / 32); ++c) {
+              uint32_t o[32];
+              tc::tmem_ld32(lane_base + kTmemO + c * 32, o);
+              tc::tmem_wait_ld();
+#pragma unroll
+              for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * f);
+              tc::tmem_st32(lane_base + kTmemO + c * 32, o);
             }
+            tc::tmem_wait_st();
           }
-          m_used = m_new;
+        }
+        if (m_own != m_used) {
+          l *= fast_exp2(m_own - m_used);  // m_used > m_own: 0 while there is no sum
+          m_own = m_used;
         }
         const float m_eff = m_used == -CUDART_INF_F ? 0.f : m_used;
-        const uint64_t sc2 = f2(sl2, sl2), nm2 = f2(-m_eff, -m_eff);
+        const uint64_t nm2 = f2(-m_eff, -m_eff);
         uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
-        uint32_t pk[32];
+#pragma unroll 1
+        for (int hf = 0; hf < opaque(2); ++hf) {
+          uint32_t sv[64], pk[32];
+          tc::tmem_ld32(s_col + hf * 64, *reinterpret_cast<uint32_t(*)[32]>(sv));
+          tc::tmem_ld32(s_col + hf * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(sv + 32));
+          tc::tmem_wait_ld();
 #pragma unroll
-        for (int e = 0; e < 32; ++e) {
-          float x0, x1;
-          unf2(ffma2(f2(__uint_as_float(s[2 * e]), __uint_as_float(s[2 * e + 1])), sc2, nm2), x0, x1);
-          const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
-          acc[e & 3] = fadd2(acc[e & 3], f2(p0, p1));
-          pk[e] = pack_bf16x2(p0, p1);
+          for (int e = 0; e < 32; ++e) {
+            float x0, x1;
+            unf2(ffma2(f2(__uint_as_float(sv[2 * e]), __uint_as_float(sv[2 * e + 1])), sc2, nm2), x0, x1);
+            const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
+            acc[e & 3] = fadd2(acc[e & 3], f2(p0, p1));
+            pk[e] = pack_bf16x2(p0, p1);
+          }
+          tc::tmem_st32(s_col + hf * 32, pk);  // over scores already read
         }
-        {
-          float a0, a1, b0, b1;
-          unf2(fadd2(acc[0], acc[1]), a0, a1);
-          unf2(fadd2(acc[2], acc[3]), b0, b1);
-          l += (a0 + a1) + (b0 + b1);
-        }
-        if (!dead) {  // P over the first 32 columns of this half's part of the S buffer
-          tc::tmem_st32(lane_base + bi * kBN + kh * 64, pk);
-          tc::tmem_wait_st();
-        }
-        const int vrows = it.klen - t * kBN;
-        if (vrows < kBN) {  // the item's last tile: clear V rows past its last visible key
-          const int st = i % v_stages;
-          if (!dead) dead = !warp_wait(&bars[B_VFULL + st], (i / v_stages) & 1, abort_flag, p.status);
-          if (!dead)
-            for (int idx = sid; idx < (kBN - vrows) * C::kHalves * 8; idx += kSoftWarps * 32) {
-              const int row = vrows + idx / (C::kHalves * 8), rem = idx % (C::kHalves * 8);
-              *reinterpret_cast<uint4*>(base + off_V + st * C::kKV + (rem >> 3) * kAtom + row * 128 + (rem & 7) * 16) =
-                  make_uint4(0u, 0u, 0u, 0u);
-            }
-          tc::fence_async_smem();
-        }
+        tc::tmem_wait_st();
         tc::fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars[B_PFULL + bi]);
+        float a0, a1, b0, b1;
+        unf2(fadd2(acc[0], acc[1]), a0, a1);
+        unf2(fadd2(acc[2], acc[3]), b0, b1);
+        l += (a0 + a1) + (b0 + b1);
+      }
+      i += it.nt;
+      if (((i ^ grp) & 1u) == 0) {  // the other group did the last tile: take this sum to its reference
+        turn_wait(quarter, i - 1);
+        const float m_last = mref[r];
+        if (m_own != m_last) l *= fast_exp2(m_own - m_last);
       }
 
-      // The item's sums to the epilogue warps (the buffer is free once they
+      // This group's sums to the epilogue warps (the buffer is free once they
       // have read the previous item's).
-      if (!dead) dead = !warp_wait(&bars[B_LFREE], (ke & 1) ^ 1, abort_flag, p.status);
-      lsum[kh * kBM + r] = l;
+      if (!dead) dead = !warp_wait_small(&bars[B_LFREE], (ke & 1) ^ 1, abort_flag);
+      lsum[grp * kBM + r] = l;
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars[B_LREADY]);
       ++ke;
@@ -660,6 +691,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncwarp();  // the producer and MMA warps reconverge after their single-lane loops
   tc::fence_before_sync();
   __syncthreads();
+  if (threadIdx.x == 0) record_abort(abort_flag, p.status);
   if (warp == kSWarp) {
     tc::fence_after_sync();
     tc::tmem_dealloc(tmem, kTmemCols);
@@ -676,16 +708,7 @@ cudaError_t launch_typed(const AttnArgs& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  // As many stages as fit, the K ring first: S runs up to three tiles ahead of
-  // P.V, so the keys are needed earlier than the values.
-  int nk = kMaxStages, nv = kMaxStages;
-  while ((nk > 2 || nv > 2) && C::smem_bytes(nk, nv) > (size_t)limit) {
-    if (nv >= nk && nv > 2)
-      --nv;
-    else
-      --nk;
-  }
-  if (C::smem_bytes(nk, nv) > (size_t)limit) return cudaErrorNotSupported;
+  if (C::kSmem > (size_t)limit) return cudaErrorNotSupported;
   CUtensorMap mq, mk, mv, mo;
   const long long kv_rows = (long long)a.B * a.Hkv * a.S_cap;
   if (!make_bf16_map(&mq, a.q, (long long)a.B * a.T, (long long)a.H * D, (long long)a.H * D, kBM) ||
@@ -694,6 +717,7 @@ cudaError_t launch_typed(const AttnArgs& a, cudaStream_t st) {
     return cudaErrorNotSupported;
   BlkParams p;
   p.seq_len = a.kv_len;
+  p.out = a.out;
   p.status = reinterpret_cast<unsigned*>(a.ws);
   p.B = a.B; p.H = a.H; p.Hkv = a.Hkv; p.T = a.T; p.S_cap = a.S_cap; p.L = a.block_L;
   p.by_L = FastDiv::make(a.block_L);
@@ -704,15 +728,12 @@ cudaError_t launch_typed(const AttnArgs& a, cudaStream_t st) {
   if ((long long)a.B * a.H * p.npb > 0x7fffffffLL) return cudaErrorNotSupported;
   p.npairs = a.B * a.H * p.npb;
   p.by_npb = FastDiv::make(p.npb);
-  p.nk = nk;
-  p.nv = nv;
   p.scale_log2 = a.scale * kLog2e;
   int G = a.max_ctas > 0 ? a.max_ctas : sm_count();
   if (G > p.npairs) G = p.npairs;
   if (G < 1) G = 1;
   if ((long long)p.npairs + G > 0x7fffffffLL) return cudaErrorNotSupported;  // a CTA's pair index steps by G
-  block_attn_kernel<D><<<(unsigned)G, kThreads, C::smem_bytes(nk, nv), st>>>(mq, mk, mv, mo, p);
-  return cudaGetLastError();
+  return launch_pdl(block_attn_kernel<D>, dim3((unsigned)G), dim3(kThreads), C::kSmem, st, mq, mk, mv, mo, p);
 }
 
 }  // namespace

@@ -158,6 +158,46 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   }
 }
 
+// The same wait in a fifth of the code (the kernels have some twenty of them,
+// and what does not fit the instruction cache is fetched again and again): on
+// giving up it only sets *abort, which must lie in shared memory, and the
+// kernel records the status once at its end (record_abort).
+__device__ __forceinline__ bool mbar_wait_small(uint64_t* bar, uint32_t parity, volatile int* abort) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .u32 t0, t1;\n\t"
+      "mov.u32 %0, 1;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "@p bra DONE;\n\t"
+      "mov.u32 t0, %%globaltimer_lo;\n"
+      "AGAIN:\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "@p bra DONE;\n\t"
+      "ld.volatile.shared.u32 t1, [%3];\n\t"
+      "setp.ne.u32 p, t1, 0;\n\t"
+      "@p bra GIVEUP;\n\t"
+      "mov.u32 t1, %%globaltimer_lo;\n\t"
+      "sub.u32 t1, t1, t0;\n\t"
+      "setp.lt.u32 p, t1, %4;\n\t"
+      "@p bra AGAIN;\n"
+      "GIVEUP:\n\t"
+      "st.volatile.shared.u32 [%3], 1;\n\t"
+      "mov.u32 %0, 0;\n"
+      "DONE:\n\t}"
+      : "=&r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity), "r"(smem_u32(const_cast<int*>(abort))), "n"((uint32_t)kWaitLimitNs)
+      : "memory");
+  return ok != 0;
+}
+// For every lane of a converged warp, with one outcome.
+__device__ __forceinline__ bool warp_wait_small(uint64_t* bar, uint32_t parity, volatile int* abort) {
+  return __all_sync(0xffffffffu, mbar_wait_small(bar, parity, abort));
+}
+// One thread, once all others are done waiting: a wait that gave up becomes the device status.
+__device__ __forceinline__ void record_abort(volatile int* abort, unsigned* status) {
+  if (*abort) record_status(status, kStatusTimeout);
+}
+
 // Waits on the phase of `bar` with `parity`, bounded by time only (used to
 // drain copies still in flight after an abort).
 __device__ inline void mbar_drain(uint64_t* bar, uint32_t parity) {

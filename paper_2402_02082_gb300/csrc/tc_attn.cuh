@@ -64,6 +64,20 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   return r;
 }
 
+// The same value, unknown to the optimizer: a loop that tests it is not copied
+// for either outcome (these kernels' time goes up with their code size: what
+// does not fit the instruction cache is fetched again on every pass).
+__device__ __forceinline__ bool opaque(bool b) {
+  int x = b ? 1 : 0;
+  asm volatile("" : "+r"(x));
+  return x != 0;
+}
+// The same for a trip count: a short loop is not unrolled.
+__device__ __forceinline__ int opaque(int n) {
+  asm volatile("" : "+r"(n));
+  return n;
+}
+
 // A shared-memory descriptor advanced by `bytes`: the start address is the
 // descriptor's low field in 16-byte units, and shared addresses stay below
 // 2^18, so the sum never carries out of it.
