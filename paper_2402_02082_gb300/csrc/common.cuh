@@ -361,6 +361,108 @@ struct CostPartition {
   }
 };
 
+// Where a share of a CostPartition starts, and its tiles.
+struct ShareStart {
+  int b, h, t0, tiles;
+};
+
+// One warp (every lane of it): the table of BatchTiles (with bt.sidx) and
+// where share x of G begins.  The caller synchronizes the block afterwards.
+// The two ends of the share are looked up by two lanes side by side, once per
+// CTA: looked up by every role of a kernel at every segment, the divisions
+// were a third of the kernel's code, and fetching code is what the start of a
+// short call waits for.
+__device__ inline void build_share(const BatchTiles& bt, const int* kv_len, int B, int H, int max_kv_len, int extra,
+                                   int TK, int G, int w, int x, ShareStart* out) {
+  const int lane = threadIdx.x & 31;
+  int start = 0, slabs = 0;  // running totals (tiles stay below 2^31)
+#pragma unroll 1
+  for (int b0 = 0; b0 < B; b0 += 32) {
+    const int b = b0 + lane;
+    int L = b < B ? kv_len[b] : 0;
+    L = L < 0 ? 0 : (L > max_kv_len ? max_kv_len : L);
+    const int nt = b < B ? (L + extra + TK - 1) / TK : 0;
+    if (b < B) {
+      bt.plen[b] = L;
+      bt.len[b] = L + extra;
+      bt.ntiles[b] = nt;
+    }
+    int ts = H * nt, ks = nt > 0 ? H : 0;  // inclusive sums over the lanes
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int a = __shfl_up_sync(0xffffffffu, ts, off), c = __shfl_up_sync(0xffffffffu, ks, off);
+      if (lane >= off) {
+        ts += a;
+        ks += c;
+      }
+    }
+    if (b < B) {
+      bt.start[b + 1] = start + ts;
+      bt.sidx[b + 1] = slabs + ks;
+    }
+    start += __shfl_sync(0xffffffffu, ts, 31);
+    slabs += __shfl_sync(0xffffffffu, ks, 31);
+  }
+  if (lane == 0) {
+    bt.start[0] = 0;
+    bt.sidx[0] = 0;
+  }
+  __syncwarp();
+  CostPartition P;
+  P.init(bt, B, H, G, w);
+  const int g = (int)P.tile_at(P.part_begin(x + (lane & 1)));
+  const int g0 = __shfl_sync(0xffffffffu, g, 0), g1 = __shfl_sync(0xffffffffu, g, 1);
+  if (lane == 0) {
+    ShareStart s = {0, 0, 0, g1 > g0 ? g1 - g0 : 0};
+    if (s.tiles > 0) {
+      int lo = 0, hi = B - 1;  // the sequence of tile g0
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if ((int)bt.start[mid] <= g0) lo = mid; else hi = mid - 1;
+      }
+      const int off = g0 - (int)bt.start[lo], nt = bt.ntiles[lo];
+      s.b = lo;
+      s.h = off / nt;
+      s.t0 = off - s.h * nt;
+    }
+    *out = s;
+  }
+}
+
+// The segments of a share in order: tiles [t0, t1) of slab (b, h).  The first
+// one starts where the share does, every other at its slab's first tile.
+struct SegWalk {
+  int b, h, t0, t1, left;  // left: tiles of the share past this segment
+  __device__ __forceinline__ void clip(const BatchTiles& bt) {
+    const int nt = bt.ntiles[b] - t0;
+    t1 = t0 + (nt < left ? nt : left);
+    left -= t1 - t0;
+  }
+  __device__ __forceinline__ void start(const BatchTiles& bt, const ShareStart& s) {
+    b = s.b;
+    h = s.h;
+    t0 = s.t0;
+    left = s.tiles;
+    clip(bt);
+  }
+  __device__ __forceinline__ bool any() const { return t1 > t0; }
+  __device__ __forceinline__ bool more() const { return left > 0; }
+  __device__ __forceinline__ bool whole(const BatchTiles& bt) const { return t0 == 0 && t1 == bt.ntiles[b]; }
+  // The next segment; without one, any() turns false.
+  __device__ __forceinline__ void next(const BatchTiles& bt, int H) {
+    if (left == 0) {
+      t0 = t1;
+      return;
+    }
+    if (++h == H) {
+      h = 0;
+      do ++b; while (bt.ntiles[b] == 0);
+    }
+    t0 = 0;
+    clip(bt);
+  }
+};
+
 // Dynamic work: the global tile sequence is cut into chunks of shrinking size
 // that CTAs claim at run time.  Level 0 holds the first half of the tiles in
 // G equal chunks, level 1 half of the rest in G chunks, and so on; the last

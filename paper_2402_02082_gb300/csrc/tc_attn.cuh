@@ -107,8 +107,8 @@ __device__ inline uint64_t ancestors(const int* parent, int n, int node, bool wa
     a[k] = x < n ? 1ull << x : 0ull;
     q[k] = (px >= 0 && px < x) ? px : -1;
   }
-#pragma unroll
-  for (int round = 0; round < 6; ++round) {
+#pragma unroll 1
+  for (int round = 0; round < opaque(6); ++round) {
     uint64_t na[2];
     int nq[2];
 #pragma unroll
@@ -128,6 +128,24 @@ __device__ inline uint64_t ancestors(const int* parent, int n, int node, bool wa
   const int v = want ? node : 0;
   const uint64_t r0 = __shfl_sync(0xffffffffu, a[0], v & 31), r1 = __shfl_sync(0xffffffffu, a[1], v & 31);
   return want ? (v < 32 ? r0 : r1) : 0ull;
+}
+
+// Zeros for the sequences without cached keys (a prefix-only call's empty
+// softmax): elements i, i + step, ... of each one's `per_seq` outputs.
+__device__ __forceinline__ void zero_empty(const BatchTiles& bt, int B, long long per_seq, float* out, int i, int step) {
+#pragma unroll 1
+  for (int b = 0; b < B; ++b)
+    if (bt.ntiles[b] == 0)
+#pragma unroll 1
+      for (long long e = i; e < per_seq; e += step) out[b * per_seq + e] = 0.f;
+}
+
+// Which of 64 consecutive keys a row sees (bit i: the i-th), the first of them
+// c0 keys past the prefix (negative: inside it): the prefix and, of the tree's
+// keys, the set `anc`, which has no bit past the tree.
+__device__ __forceinline__ uint64_t visible_keys(uint64_t anc, int c0) {
+  if (c0 >= 0) return c0 < 64 ? anc >> c0 : 0ull;
+  return c0 > -64 ? (anc << -c0) | ((1ull << -c0) - 1ull) : ~0ull;
 }
 
 // Merges the partials of every split slab: one warp per query row r of slab

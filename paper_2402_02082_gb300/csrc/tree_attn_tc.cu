@@ -112,7 +112,7 @@ struct TcCfg {
   static __host__ __device__ uint32_t off_bar(int ns) { return off_V(ns) + ns * kKVTile; }
   static __host__ __device__ uint32_t off_ml(int ns) { return off_bar(ns) + 512; }
   static __host__ __device__ uint32_t off_misc(int ns) { return off_ml(ns) + 2 * kM * 8; }
-  static __host__ __device__ uint32_t off_tab(int ns) { return off_misc(ns) + 48; }
+  static __host__ __device__ uint32_t off_tab(int ns) { return off_misc(ns) + 48; }  // misc: TMEM slot, abort flag, share start
   static constexpr uint32_t kTmemO = kSBuf * kTK;                  // S buffers at columns 0, 64, 128, 192
   static constexpr uint32_t kTmemCols = kTmemO + 2 * D <= 256 ? 256 : 512;
   static_assert(kTmemO + 2 * D <= 512, "TMEM columns");
@@ -157,6 +157,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   float2* ml = reinterpret_cast<float2*>(base + C::off_ml(ns));
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + C::off_misc(ns));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(base + C::off_misc(ns) + 4);
+  ShareStart* share = reinterpret_cast<ShareStart*>(base + C::off_misc(ns) + 16);
   BatchTiles bt;
   bt.start = reinterpret_cast<long long*>(base + C::off_tab(ns));
   bt.len = reinterpret_cast<int*>(bt.start + p.B + 1);
@@ -188,16 +189,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc::tmem_relinquish();
   }
   tc::fence_before_sync();
-  build_batch_tiles(bt, p.kv_len, p.B, p.Hkv, p.max_kv_len, p.tree ? n : 0, kTK);  // __syncthreads inside
+  // this CTA: share x of the key sequence, row tile y of every slab in it;
+  // shares of equal cost, a segment switch counted as seg_weight tiles
+  const int G = gridDim.x / p.R, x = blockIdx.x / p.R, y = blockIdx.x - x * p.R;
+  const int row0 = y * kM, rows_here = min(kM, p.rows - row0);
+  const int weight = seg_weight(p.rows < kM ? p.rows : kM);
+  if (warp == 0) build_share(bt, p.kv_len, p.B, p.Hkv, p.max_kv_len, p.tree ? n : 0, kTK, G, weight, x, share);
+  __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = *tmem_slot;
 
-  // this CTA: share x of the key sequence, row tile y of every slab in it
-  const int x = blockIdx.x / p.R, y = blockIdx.x - x * p.R;
-  const int row0 = y * kM, rows_here = min(kM, p.rows - row0);
-  CostPartition P;  // shares of equal cost, a segment switch counted as seg_weight tiles
-  P.init(bt, p.B, p.Hkv, gridDim.x / p.R, seg_weight(p.rows < kM ? p.rows : kM));
-  const long long g_begin = P.begin(x), g_end = P.end(x);
+  SegWalk s;
+  s.start(bt, *share);
 
   if (warp == kProdWarp || warp == kVProdWarp) {
     // ----------------------------------------------------------- producers
@@ -215,88 +218,99 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t dst0 = is_k ? C::off_K : off_V;
       // one reader per tile: evict it first; R row tiles read each tile R times
       const uint64_t pol = p.R == 1 ? policy_evict_first() : policy_evict_normal();
-      int i = 0;
+      int issued = 0, st = 0;
+      uint32_t phase = 1;
       bool ok = true;
-      for (long long g = g_begin; g < g_end && ok;) {
-        const Segment sg = locate(bt, P, p.B, g, g_end);
-        const int row0k = (sg.b * p.Hkv + sg.h) * p.S_cap;
-        for (int t = sg.t0; t < sg.t1; ++t, ++i) {
-          const int st = i % ns;
-          if (!mbar_wait(&empty[st], ((i / ns) & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
+      for (; s.any() && ok; s.next(bt, p.Hkv)) {
+        int row = (s.b * p.Hkv + s.h) * p.S_cap + s.t0 * kTK;
+        for (int t = s.t0; t < s.t1; ++t, row += kTK) {
+          ok = mbar_wait_small(&empty[st], phase, abort_flag);
+          if (!ok) break;
           mbar_arrive_expect_tx(&full[st], C::kKVTile);
           for (int hd = 0; hd < C::kHalves; ++hd)
-            tc::tma_load_2d(base + dst0 + st * C::kKVTile + hd * C::kKVHalf, map, hd * 64, row0k + t * kTK, &full[st],
-                            pol);
+            tc::tma_load_2d(base + dst0 + st * C::kKVTile + hd * C::kKVHalf, map, hd * 64, row, &full[st], pol);
+          ++issued;
+          if (++st == ns) {
+            st = 0;
+            phase ^= 1;
+          }
         }
-        g = sg.g_end;
       }
       if (!ok)  // aborted: let issued loads land before the CTA exits
-        for (int j = (i > ns ? i - ns : 0); j < i; ++j) mbar_drain(&full[j % ns], (j / ns) & 1);
+        for (int j = (issued > ns ? issued - ns : 0); j < issued; ++j) mbar_drain(&full[j % ns], (j / ns) & 1);
     }
   } else if (warp >= kMmaWarp) {  // warps 9-11
     // ----------------------------------------------------------- MMA issue
     const int role = warp - kMmaWarp;  // 0, 1: S of tiles with j % 2 == role; 2: P.V
     if (lane == 0) {
-      constexpr uint32_t idS = tc::idesc_bf16_f32(kM, kTK, false, false);
-      constexpr uint32_t idO = tc::idesc_bf16_f32(kM, D, false, true);
-      const uint32_t sQ = smem_u32(base + C::off_Q), sP = smem_u32(base + C::off_P);
-      const uint32_t sK = smem_u32(base + C::off_K), sV = smem_u32(base + off_V);
-      int i = 0, seg = 0;
+      // Ring positions are counted, not divided out.
       bool ok = true;
-      // S(j) = Q K(j)^T into S buffer j % kSBuf
-      auto issue_s = [&](int j) -> bool {
-        if (!mbar_wait(&bars[B_KFULL + j % ns], (j / ns) & 1, abort_flag, p.status) ||
-            !mbar_wait(&bars[B_SFREE + j % kSBuf], ((j / kSBuf) & 1) ^ 1, abort_flag, p.status))
-          return false;
-        tc::fence_after_sync();
-        const uint32_t kb = sK + (j % ns) * C::kKVTile;
+      if (role < 2) {
+        // S(j) = Q K(j)^T into S buffer j % kSBuf, for the tiles j with j % 2 ==
+        // role; Q of the segment must be in place first
+        constexpr uint32_t idS = tc::idesc_bf16_f32(kM, kTK, false, false);
+        const uint64_t dQ = tc::sw128_desc(smem_u32(base + C::off_Q), 16, 1024);
+        const uint64_t dK0 = tc::sw128_desc(smem_u32(base + C::off_K), 16, 1024);
+        int i = 0, seg = 0, st = role, bi = role;
+        uint32_t k_phase = 0, s_phase = 1;
+        for (; s.any() && ok; s.next(bt, p.Hkv), ++seg) {
+          bool q_ready = false;
+          for (int t = s.t0; t < s.t1; ++t, ++i) {
+            if ((i & 1) != role) continue;
+            ok = (q_ready || mbar_wait_small(&bars[B_QFULL + (seg & 1)], (seg >> 1) & 1, abort_flag)) &&
+                 mbar_wait_small(&bars[B_KFULL + st], k_phase, abort_flag) &&
+                 mbar_wait_small(&bars[B_SFREE + bi], s_phase, abort_flag);
+            if (!ok) break;
+            q_ready = true;
+            tc::fence_after_sync();
+            const uint64_t dK = dK0 + (uint64_t)st * desc_step(C::kKVTile);
 #pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-          const uint64_t a = tc::sw128_desc(sQ + (ks / 4) * C::kQHalf + (ks % 4) * 32, 16, 1024);
-          const uint64_t bdesc = tc::sw128_desc(kb + (ks / 4) * C::kKVHalf + (ks % 4) * 32, 16, 1024);
-          tc::mma_bf16(tmem + (j % kSBuf) * kTK, a, bdesc, idS, ks > 0 ? 1u : 0u);
-        }
-        tc::mma_commit(&bars[B_SFULL + j % kSBuf]);
-        tc::mma_commit(&bars[B_KEMPTY + j % ns]);
-        return true;
-      };
-      // O_h += P[:, 32h .. 32h+31] V[32h .. 32h+31, :] for key halves h = 0, 1
-      auto issue_pv = [&](int jj, bool first_in_seg) -> bool {
-        if (!mbar_wait(&bars[B_PFULL + (jj & 1)], (jj >> 1) & 1, abort_flag, p.status)) return false;
-        if (!mbar_wait(&bars[B_VFULL + jj % ns], (jj / ns) & 1, abort_flag, p.status)) return false;
-        if (first_in_seg && seg > 0 && !mbar_wait(&bars[B_OFREE], (seg - 1) & 1, abort_flag, p.status)) return false;
-        tc::fence_after_sync();
-        const uint32_t vb = sV + (jj % ns) * C::kKVTile;
-        const uint32_t pb = sP + (jj & 1) * C::kPBytes;
-#pragma unroll
-        for (int ks = 0; ks < kTK / 16; ++ks) {
-          const int h = ks >> 1;
-          const uint64_t a = tc::sw128_desc(pb + ks * 32, 16, 1024);
-          const uint64_t bdesc = tc::sw128_desc(vb + ks * 16 * 128, C::kKVHalf, 1024);
-          tc::mma_bf16(tmem + C::kTmemO + h * D, a, bdesc, idO, (first_in_seg && (ks & 1) == 0) ? 0u : 1u);
-        }
-        tc::mma_commit(&bars[B_PFREE + (jj & 1)]);
-        tc::mma_commit(&bars[B_VEMPTY + jj % ns]);
-        tc::mma_commit(&bars[B_ODONE + (jj & 3)]);
-        return true;
-      };
-      for (long long g = g_begin; g < g_end && ok;) {
-        const Segment s = locate(bt, P, p.B, g, g_end);
-        if (role < 2) {
-          // S of the tiles j with j % 2 == role; Q of the segment must be in place first
-          const int ntile = s.t1 - s.t0;
-          const bool mine = ntile > 1 || (i & 1) == role;
-          if (mine && !mbar_wait(&bars[B_QFULL + (seg & 1)], (seg >> 1) & 1, abort_flag, p.status)) {
-            ok = false;
-            break;
+            for (int ks = 0; ks < D / 16; ++ks)
+              tc::mma_bf16(tmem + bi * kTK, dQ + desc_step((ks / 4) * C::kQHalf + (ks % 4) * 32),
+                           dK + desc_step((ks / 4) * C::kKVHalf + (ks % 4) * 32), idS, ks > 0 ? 1u : 0u);
+            tc::mma_commit(&bars[B_SFULL + bi]);
+            tc::mma_commit(&bars[B_KEMPTY + st]);
+            if ((st += 2) >= ns) {
+              st = role;
+              k_phase ^= 1;
+            }
+            if ((bi += 2) >= kSBuf) {
+              bi = role;
+              s_phase ^= 1;
+            }
           }
-          for (int t = s.t0; t < s.t1 && ok; ++t, ++i)
-            if ((i & 1) == role) ok = issue_s(i);
-        } else {
-          for (int t = s.t0; t < s.t1 && ok; ++t, ++i) ok = issue_pv(i, t == s.t0);
         }
-        ++seg;
-        g = s.g_end;
+      } else {
+        // O_h += P[:, 32h .. 32h+31] V[32h .. 32h+31, :] for key halves h = 0, 1
+        constexpr uint32_t idO = tc::idesc_bf16_f32(kM, D, false, true);
+        const uint64_t dP0 = tc::sw128_desc(smem_u32(base + C::off_P), 16, 1024);
+        const uint64_t dV0 = tc::sw128_desc(smem_u32(base + off_V), C::kKVHalf, 1024);
+        int i = 0, seg = 0, st = 0;
+        uint32_t v_phase = 0;
+        for (; s.any() && ok; s.next(bt, p.Hkv), ++seg) {
+          if (seg > 0) ok = mbar_wait_small(&bars[B_OFREE], (seg - 1) & 1, abort_flag);
+          uint32_t acc = 0;
+          for (int t = s.t0; t < s.t1 && ok; ++t, ++i) {
+            ok = mbar_wait_small(&bars[B_VFULL + st], v_phase, abort_flag) &&
+                 mbar_wait_small(&bars[B_PFULL + (i & 1)], (i >> 1) & 1, abort_flag);
+            if (!ok) break;
+            tc::fence_after_sync();
+            const uint64_t dV = dV0 + (uint64_t)st * desc_step(C::kKVTile);
+            const uint64_t dP = dP0 + (uint64_t)(i & 1) * desc_step(C::kPBytes);
+#pragma unroll
+            for (int ks = 0; ks < kTK / 16; ++ks)
+              tc::mma_bf16(tmem + C::kTmemO + (ks >> 1) * D, dP + desc_step(ks * 32), dV + desc_step(ks * 16 * 128), idO,
+                           (ks & 1) == 0 ? acc : 1u);
+            acc = 1;
+            tc::mma_commit(&bars[B_PFREE + (i & 1)]);
+            tc::mma_commit(&bars[B_VEMPTY + st]);
+            tc::mma_commit(&bars[B_ODONE + (i & 3)]);
+            if (++st == ns) {
+              st = 0;
+              v_phase ^= 1;
+            }
+          }
+        }
       }
       tc::mma_commit(&bars[B_MDONE + role]);  // every MMA finished before TMEM is released
       mbar_drain(&bars[B_MDONE + role], 0);
@@ -318,22 +332,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int sid = threadIdx.x;                  // 0..255 among the softmax threads
     const float sl2 = p.scale_log2;
     bool dead = false;
-    int i = 0, seg = 0;
+    int i = 0, seg = 0, vst = 0;  // tiles, segments, V stage and its phase
+    uint32_t v_phase = 0;
     // Segment sg's queries into the swizzled Q tile (padding rows are zero);
     // the two threads of a row write chunks 0-3 and 4-7 of each 128-byte atom.
     // Key-half-0 warps only.
     const OutMap om{p.group, p.H};
-    // this thread's query row of slab (sb, h): its row in q / out (-1: none),
-    // and the prefix keys it sees (< lim)
-    auto row_at = [&](const Segment& sq, int& lim) -> long long {
-      lim = bt.plen[sq.b];
-      if (!valid) return -1;
-      return om.row(sq.b, sq.h, row0 + qi, p.rows);
+    // this thread's query row of the segment's slab in q / out (-1: none)
+    auto row_at = [&](const SegWalk& sq) -> long long {
+      return valid ? om.row(sq.b, sq.h, row0 + qi, p.rows) : -1;
     };
-    auto write_q = [&](const Segment& sq, int sg) {
+    auto write_q = [&](const SegWalk& sq, int sg) {
       unsigned char* qrow = base + C::off_Q + (row >> 3) * 1024 + (row & 7) * 128;
-      int lim_unused;
-      const long long qr = row_at(sq, lim_unused);
+      const long long qr = row_at(sq);
       const uint4* src = reinterpret_cast<const uint4*>(p.q + (qr >= 0 ? qr : 0) * D);
 #pragma unroll
       for (int hd = 0; hd < C::kHalves; ++hd)
@@ -349,14 +360,17 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (lane == 0) mbar_arrive(&bars[B_QFULL + (sg & 1)]);
     };
     // The first segment's queries first: the first S products wait for them.
-    if (half == 0 && g_begin < g_end) write_q(locate(bt, P, p.B, g_begin, g_end), 0);
+    if (half == 0 && s.any()) write_q(s, 0);
     // Then, off the path to the first S products: the share range of every
     // slab split over several shares, for the merge kernel ((-1, -1): written
     // out directly, or no keys), and zeros for a prefix-only call's sequences
     // without cached keys (an empty softmax).
     constexpr int kST = kSoftWarps * 32;
-    if (y == 0)
-      for (int bh = x * kST + (int)threadIdx.x; bh < p.B * p.Hkv; bh += (gridDim.x / p.R) * kST) {
+    if (y == 0) {
+      CostPartition P;
+      P.init(bt, p.B, p.Hkv, G, weight);
+#pragma unroll 1
+      for (int bh = x * kST + (int)threadIdx.x; bh < p.B * p.Hkv; bh += G * kST) {
         const int b = bh / p.Hkv, nt = bt.ntiles[b];
         int2 r = make_int2(-1, -1);
         if (nt > 0) {
@@ -366,16 +380,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         p.ranges[bh] = r;
       }
-    if (!p.tree) {
-      const long long total = (long long)p.B * n * p.H * D;
-      for (long long idx = (long long)blockIdx.x * kST + threadIdx.x; idx < total; idx += (long long)gridDim.x * kST)
-        if (bt.ntiles[idx / ((long long)n * p.H * D)] == 0) p.out[idx] = 0.f;
     }
-    for (long long g = g_begin; g < g_end; ++seg) {
-      const Segment s = locate(bt, P, p.B, g, g_end);
+    if (!p.tree) zero_empty(bt, p.B, (long long)n * p.H * D, p.out, (int)blockIdx.x * kST + (int)threadIdx.x, (int)gridDim.x * kST);
+    for (; s.any(); s.next(bt, p.Hkv), ++seg) {
       const int plen = bt.plen[s.b], len = bt.len[s.b];
-      int rowlim;  // keys below it are visible to this row (the prefix)
-      const long long orow = row_at(s, rowlim);
+      const long long orow = row_at(s);
 
       // the ancestor-or-self set of this row's tree node, found when the first
       // tile with tree keys comes (prefix only: no tree keys)
@@ -386,11 +395,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       // S of the next tile is loaded while this tile's exponentials run (within
       // the segment only: the next segment's S needs a Q written after it ends)
       uint32_t sr[16];
-      if (!dead) dead = !warp_wait(&bars[B_SFULL + i % kSBuf], (i / kSBuf) & 1, abort_flag, p.status);
-      if (!dead) {
-        tc::fence_after_sync();
-        tc::tmem_ld16x64b_x16(lane_addr + (i % kSBuf) * kTK + half * kHK, sr);
-      }
+      if (!dead) dead = !warp_wait_small(&bars[B_SFULL + i % kSBuf], (i / kSBuf) & 1, abort_flag);
+      tc::fence_after_sync();
+      tc::tmem_ld16x64b_x16(lane_addr + (i % kSBuf) * kTK + half * kHK, sr);
       for (int t = s.t0; t < s.t1; ++t, ++i) {
         const int j = i;
         tc::tmem_wait_ld();
@@ -411,24 +418,20 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int k = 0; k < 16; ++k) sc[k] = __uint_as_float(cur[k]) * sl2;
         } else {
-          if (!anc_ready) {  // warp-uniform: t, half and plen are the same in every lane
+          if (!opaque(anc_ready)) {  // warp-uniform: t, half and plen are the same in every lane
             anc = ancestors(p.parent + (size_t)s.b * n, n, node, valid, lane);
             anc_ready = true;
           }
+          const uint32_t vis = (uint32_t)visible_keys(anc, key0 - plen);
 #pragma unroll
-          for (int k = 0; k < 16; ++k) {
-            const int key = key0 + 2 * k;
-            const bool vis = key < rowlim || (key < len && ((anc >> ((key - plen) & 63)) & 1ull));
-            sc[k] = vis ? __uint_as_float(cur[k]) * sl2 : -CUDART_INF_F;
-          }
+          for (int k = 0; k < 16; ++k)
+            sc[k] = (vis & (1u << 2 * k)) ? __uint_as_float(cur[k]) * sl2 : -CUDART_INF_F;
         }
         if (t + 1 < s.t1) {  // start loading S of the next tile
           const int jn = j + 1;
-          if (!dead) dead = !warp_wait(&bars[B_SFULL + jn % kSBuf], (jn / kSBuf) & 1, abort_flag, p.status);
-          if (!dead) {
-            tc::fence_after_sync();
-            tc::tmem_ld16x64b_x16(lane_addr + (jn % kSBuf) * kTK + half * kHK, sr);
-          }
+          if (!opaque(dead)) dead = !warp_wait_small(&bars[B_SFULL + jn % kSBuf], (jn / kSBuf) & 1, abort_flag);
+          tc::fence_after_sync();
+          tc::tmem_ld16x64b_x16(lane_addr + (jn % kSBuf) * kTK + half * kHK, sr);
         }
         float mx[4] = {sc[0], sc[1], sc[2], sc[3]};
 #pragma unroll
@@ -442,11 +445,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           const float f = need ? fast_exp2(m_used - m_new) : 1.f;
           l *= f;
           if (t > s.t0 && !dead) {  // O holds the P.V of earlier tiles of this segment
-            dead = !warp_wait(&bars[B_ODONE + ((j - 1) & 3)], ((j - 1) >> 2) & 1, abort_flag, p.status);
+            dead = !warp_wait_small(&bars[B_ODONE + ((j - 1) & 3)], ((j - 1) >> 2) & 1, abort_flag);
             if (!dead) {
               tc::fence_after_sync();
 #pragma unroll 1
-              for (int c = 0; c < D / 32; ++c) {
+              for (int c = 0; c < opaque(D / 32); ++c) {
                 uint32_t o[16];
                 tc::tmem_ld16x64b_x16(lane_addr + o_col + c * 32, o);
                 tc::tmem_wait_ld();
@@ -478,7 +481,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           pk[k] = cpar ? pack_bf16x2(recv, pv[8 + k]) : pack_bf16x2(pv[k], recv);
         }
 
-        if (!dead) dead = !warp_wait(&bars[B_PFREE + (j & 1)], ((j >> 1) & 1) ^ 1, abort_flag, p.status);
+        if (!opaque(dead)) dead = !warp_wait_small(&bars[B_PFREE + (j & 1)], ((j >> 1) & 1) ^ 1, abort_flag);
         {
           unsigned char* prow = base + C::off_P + (j & 1) * C::kPBytes + (row >> 3) * 1024 + (row & 7) * 128;
 #pragma unroll
@@ -490,11 +493,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         const int vrows = len - t * kTK;
         if (vrows < kTK) {  // last tile of the slab: clear V rows past its end
-          const int st = j % ns;
-          if (!dead) dead = !warp_wait(&bars[B_VFULL + st], (j / ns) & 1, abort_flag, p.status);
+          if (!dead) dead = !warp_wait_small(&bars[B_VFULL + vst], v_phase, abort_flag);
+#pragma unroll 1
           for (int idx = sid; idx < (kTK - vrows) * C::kHalves; idx += kSoftWarps * 32) {
             const int r = vrows + idx / C::kHalves, hd = idx % C::kHalves;
-            uint4* dst = reinterpret_cast<uint4*>(base + off_V + st * C::kKVTile + hd * C::kKVHalf + r * 128);
+            uint4* dst = reinterpret_cast<uint4*>(base + off_V + vst * C::kKVTile + hd * C::kKVHalf + r * 128);
 #pragma unroll
             for (int c = 0; c < 8; ++c) dst[c] = make_uint4(0u, 0u, 0u, 0u);
           }
@@ -503,12 +506,20 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc::fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars[B_PFULL + (j & 1)]);
+        if (++vst == ns) {
+          vst = 0;
+          v_phase ^= 1;
+        }
       }
 
       // Every S product of this segment has been consumed, so Q is free: write
       // the next segment's queries now and let its S products overlap this
       // epilogue.
-      if (half == 0 && s.g_end < g_end) write_q(locate(bt, P, p.B, s.g_end, g_end), seg + 1);
+      if (half == 0 && s.more()) {
+        SegWalk nx = s;
+        nx.next(bt, p.Hkv);
+        write_q(nx, seg + 1);
+      }
 
       // ---- segment epilogue: merge the two key halves, then O / l or a split
       // partial.  Each half writes half of the head dims, reading both halves'
@@ -523,14 +534,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       ml_sync();
       {
         const int jl = i - 1;
-        if (!dead) dead = !warp_wait(&bars[B_ODONE + (jl & 3)], (jl >> 2) & 1, abort_flag, p.status);
+        if (!dead) dead = !warp_wait_small(&bars[B_ODONE + (jl & 3)], (jl >> 2) & 1, abort_flag);
         const float m0 = half == 0 ? m_used : other.x, l0 = half == 0 ? l : other.y;
         const float m1 = half == 0 ? other.x : m_used, l1 = half == 0 ? other.y : l;
         const float M = fmaxf(m0, m1);
         const float f0 = m0 == -CUDART_INF_F ? 0.f : fast_exp2(m0 - M);
         const float f1 = m1 == -CUDART_INF_F ? 0.f : fast_exp2(m1 - M);
         const float L = l0 * f0 + l1 * f1;
-        const bool single = s.c_first == s.c_last;
+        const bool single = s.whole(bt);  // the whole slab in this share
         const int bh = s.b * p.Hkv + s.h;
         float* dst = single ? p.out + (orow >= 0 ? orow : 0) * D
                             : partial_slot(p.partials, x + bh, p.rows, D) + (size_t)(row0 + (valid ? qi : 0)) * (D + 2) + 2;
@@ -585,13 +596,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars[B_OFREE]);
       }
-      g = s.g_end;
     }
   }
 
   __syncwarp();  // the producer and MMA warps reconverge after their single-lane loops
   tc::fence_before_sync();
   __syncthreads();
+  if (threadIdx.x == 0) record_abort(abort_flag, p.status);
   if (warp == kMmaWarp) {
     tc::fence_after_sync();
     tc::tmem_dealloc(tmem, C::kTmemCols);
