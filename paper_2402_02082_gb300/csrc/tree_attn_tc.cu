@@ -48,6 +48,17 @@
 // V rows past the end of a slab are zeroed in shared memory before P.V (the
 // cache beyond kv_len + n may hold anything, even NaN).
 //
+// Code size.  A short call's time is mostly its start: the CTAs fetch their code
+// from L2 while the first keys are in flight, so every role's code lies on the
+// path to the first result.  The share is looked up once per CTA (build_share)
+// and walked without divisions, ring positions are counted, waits are small and
+// the tree mask comes from one shifted window of the ancestor set: 92 KB of code
+// became 59 KB, batch-1 Vicuna-7B (2048 keys, 6 nodes) 17.7 -> 16.0 us, the
+// ragged Vicuna-13B batch (8 x 40 heads, 512-4096 keys, 26 nodes) 79.1 -> 72.2,
+// 3 x 40 heads of D = 64 with up to 441 keys 14.7 -> 12.1.  Long contexts, where
+// the stream is the bound, did not change (4 x 52 heads, 16384 keys: 282 us over
+// rotating caches).
+//
 // A slab whose keys fall in one CTA's share is written out directly.  A slab
 // split over several shares leaves one partial (max, sum, o) per share in the
 // workspace, and the kernel records the slab's share range; a second kernel,
