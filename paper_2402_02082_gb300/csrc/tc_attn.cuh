@@ -20,19 +20,6 @@ __device__ __forceinline__ uint64_t policy_evict_last() {
   return p;
 }
 
-// Warp-uniform bounded wait: every lane probes once and the warp votes; only
-// if the phase is not complete yet does lane 0 run the bounded wait and the
-// warp follow it.  Every lane sees the same outcome, so the warp-collective
-// tcgen05 instructions after it stay convergent.
-__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort, unsigned* status) {
-  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-  int ok = 1;
-  if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, abort, status) ? 1 : 0;
-  ok = __shfl_sync(0xffffffffu, ok, 0);
-  __syncwarp();
-  return ok != 0;
-}
-
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   uint32_t r;
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));

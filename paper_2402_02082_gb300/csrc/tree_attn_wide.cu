@@ -14,17 +14,25 @@
 // while the bytes stay the same.  Here a row tile is 128 rows and a key tile
 // 128 keys, the shape of the training-time block-mask kernel:
 //   S = Q K^T : M = 128 query rows, N = 128 keys, K = D, operands in shared memory
-//   O += P V  : M = 128, N = D, K = 64 keys per key half, P in tensor memory
+//   O += P V  : M = 128, N = D, K = 128 keys, P in tensor memory
 // which does four times the (row, key) pairs of a 64 x 64 tile per softmax
-// pass; at one row tile that leaves the loop ~20% faster than the HBM pace of
-// an SM, where the 64-row kernel's loop runs right at it, so grouped-query
-// slabs of few rows come here too.  Tensor memory holds three S buffers of
-// 128 columns (S of tile i + 3 waits for P.V of tile i) and the O
-// accumulator.  Two softmax groups of four
-// warps take the two 64-key halves of every tile, one thread per row; the two
-// threads of a row agree on each tile's row max through one TMEM column, so
-// both halves use one reference max and accumulate into the one O, and each
-// group writes P over the first 32 columns of its half of the S buffer.
+// pass.  Tensor memory holds three S buffers of 128 columns (S of tile i + 3
+// waits for P.V of tile i) and the O accumulator.  Two softmax groups of four
+// warps take the tiles in turn, one thread per row: the softmax of a tile is a
+// serial chain of ~1500 cycles and each group has two tile periods for it.  The
+// reference max of the online softmax passes from tile to tile, so from group
+// to group, through shared memory; a group keeps its own row sum and takes it
+// to the segment's last reference at the end.  P overwrites the first 64
+// columns of its S buffer.
+//
+// Code size counts like a resource here (see the 64-row kernel): the loops are
+// rolled 64 scores at a time, the share is looked up once per CTA, waits are
+// small: 99 KB of code became 52 KB.  Measured on Mistral-7B's 32 over 8 heads
+// (16384 keys, 4 sequences): the 33-node tree, two row tiles (132 rows of 256),
+// 72.4 -> 62.7 us; the draft step, 4 rows, 48.1 -> 46.2; 2 sequences of 211
+// keys, one node, 11.2 -> 8.9; one sequence of 13645 keys, 3 nodes, 21.9 -> 18.7
+// (before: the groups on the two key halves of every tile, meeting in an
+// exchange of the row max).
 //
 // Work: the slabs' 128-key tiles are cut into G shares of equal cost (a
 // segment switch counted as kSegWeight tiles), and R = ceil(rows / 128)
@@ -43,12 +51,11 @@
 //
 // Roles (384 threads, one CTA per SM):
 //   warps 0-7  softmax and the segment epilogues: warp w reads TMEM lane
-//              quarter w % 4 (one thread per row) and key half w / 4.
-//   warp 8     lane 0: the queries of each segment and the K ring (2-D TMA,
-//              128-byte swizzle), polling both.
-//   warp 9     S issue (lane 0) and the TMEM allocation.
+//              quarter w % 4 (one thread per row) of the tiles of parity w / 4.
+//   warp 8     the K ring, warp 11 the V ring (2-D TMA by lane 0, 128-byte
+//              swizzle); warp 11's lanes clear the V rows past a slab's end.
+//   warp 9     lane 0: the queries of each segment, S issue; the TMEM allocation.
 //   warp 10    P.V issue (lane 0).
-//   warp 11    lane 0: the V ring.
 //
 // Masking: keys below the sequence's prefix length are visible to every row;
 // tree key c (at prefix + c) is visible to the rows of node i iff c is an
@@ -75,9 +82,9 @@ namespace {
 constexpr int kBM = 128;          // query rows per row tile (MMA rows, TMEM lanes)
 constexpr int kBN = 128;          // keys per tile
 constexpr int kMaxStages = 4;     // K/V ring stages (the launch picks as many as fit)
-constexpr int kSoftWarps = 8;     // two groups of four: the key halves of every tile
-constexpr int kKProdWarp = 8;     // the queries and the K ring
-constexpr int kSWarp = 9;
+constexpr int kSoftWarps = 8;     // two groups of four: the even and the odd tiles
+constexpr int kKProdWarp = 8;     // the K ring
+constexpr int kSWarp = 9;         // the queries and S
 constexpr int kPVWarp = 10;
 constexpr int kVProdWarp = 11;
 constexpr int kThreads = 384;
@@ -98,7 +105,7 @@ constexpr int kSegWeight = 4;
 // the completion of tile i - 2 (measured: the last tiles of a segment missing
 // from O when the values arrived late from DRAM).
 constexpr int B_KFULL = 0, B_KEMPTY = 4, B_VFULL = 8, B_VEMPTY = 12, B_QFULL = 16, B_QEMPTY = 17, B_SFULL = 18,
-              B_PFULL = 21, B_BFREE = 24, B_ODONE = 27, B_MDONE = 31, kNumBars = 33;
+              B_PFULL = 21, B_BFREE = 24, B_ODONE = 27, B_MDONE = 31, B_OFREE = 33, B_VCLR = 34, kNumBars = 38;
 
 template <int D>
 struct WideCfg {
@@ -110,15 +117,17 @@ struct WideCfg {
   // K ring of nk stages, then the V ring of nv, barriers, misc, row sums, batch table
   static __host__ __device__ uint32_t off_V(int nk) { return off_K + nk * kKV; }
   static __host__ __device__ uint32_t off_bar(int nk, int nv) { return off_V(nk) + nv * kKV; }
-  static __host__ __device__ uint32_t off_misc(int nk, int nv) { return off_bar(nk, nv) + 512; }
-  // the segment's row sums, [key half][row], between the two softmax groups
-  static __host__ __device__ uint32_t off_lsum(int nk, int nv) { return off_misc(nk, nv) + 16; }
-  static __host__ __device__ uint32_t off_tab(int nk, int nv) { return off_lsum(nk, nv) + 2 * kBM * 4; }
+  // TMEM slot, abort flag, share start
+  static __host__ __device__ uint32_t off_misc(int nk, int nv) { return off_bar(nk, nv) + kNumBars * 8; }
+  // [2][row]: during a segment, [0] holds the running reference max of every
+  // row; at its end, both hold the groups' row sums
+  static __host__ __device__ uint32_t off_row(int nk, int nv) { return off_misc(nk, nv) + 32; }
+  static __host__ __device__ uint32_t off_tab(int nk, int nv) { return off_row(nk, nv) + 2 * kBM * 4; }
   static size_t smem_bytes(int B, int nk, int nv) {
     return 1024 + off_tab(nk, nv) + (size_t)(B + 1) * 8 + (size_t)(4 * B + 1) * 4;
   }
   static_assert(kTmemO + D <= kTmemCols, "TMEM columns");
-  static_assert(kNumBars * 8 <= 512, "barrier area");
+  static_assert(kNumBars % 2 == 0, "alignment");
 };
 
 struct WideParams {
@@ -136,6 +145,16 @@ struct WideParams {
   float scale_log2;
 };
 
+// The hand-over of a tile's reference max between the two warps (one of each
+// softmax group) of a TMEM lane quarter: named barriers 8-15, per quarter and
+// tile parity; the tile's warp arrives, the next tile's warp waits.
+__device__ __forceinline__ void turn_pass(int quarter, unsigned tile) {
+  asm volatile("bar.arrive %0, 64;" ::"r"(8 + 2 * quarter + (int)(tile & 1)) : "memory");
+}
+__device__ __forceinline__ void turn_wait(int quarter, unsigned tile) {
+  asm volatile("bar.sync %0, 64;" ::"r"(8 + 2 * quarter + (int)(tile & 1)) : "memory");
+}
+
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
     tree_attn_wide_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -148,7 +167,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* bars = reinterpret_cast<uint64_t*>(base + C::off_bar(nk, nv));
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + C::off_misc(nk, nv));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(base + C::off_misc(nk, nv) + 4);
-  float* lsum = reinterpret_cast<float*>(base + C::off_lsum(nk, nv));
+  ShareStart* share = reinterpret_cast<ShareStart*>(base + C::off_misc(nk, nv) + 16);
+  float* rowbuf = reinterpret_cast<float*>(base + C::off_row(nk, nv));
   BatchTiles bt;
   bt.start = reinterpret_cast<long long*>(base + C::off_tab(nk, nv));
   bt.len = reinterpret_cast<int*>(bt.start + p.B + 1);
@@ -163,7 +183,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc::prefetch_tmap(&tmQ);
     tc::prefetch_tmap(&tmK);
     tc::prefetch_tmap(&tmV);
-    for (int b = 0; b < kNumBars; ++b) mbar_init(&bars[b], (b >= B_PFULL && b < B_PFULL + kSBufs) ? kSoftWarps : 1);
+#pragma unroll 1
+    for (int b = 0; b < kNumBars; ++b)
+      mbar_init(&bars[b], b >= B_PFULL && b < B_PFULL + kSBufs ? kSoftWarps / 2 : b == B_OFREE ? kSoftWarps : 1);
     *abort_flag = 0;
     fence_barrier_init();
   }
@@ -173,179 +195,177 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc::tmem_relinquish();
   }
   tc::fence_before_sync();
-  build_batch_tiles(bt, p.kv_len, p.B, p.Hkv, p.max_kv_len, p.tree ? p.n : 0, kBN);  // __syncthreads inside
+  // this CTA: share x of the key tiles, row tile y of every slab in it
+  const int G = gridDim.x / p.R, x = blockIdx.x / p.R, y = blockIdx.x - x * p.R;
+  const int row0 = y * kBM;
+  if (warp == 0) build_share(bt, p.kv_len, p.B, p.Hkv, p.max_kv_len, p.tree ? p.n : 0, kBN, G, kSegWeight, x, share);
+  __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = *tmem_slot;
+  SegWalk s;
+  s.start(bt, *share);
 
-  // this CTA: share x of the key tiles, row tile y of every slab in it
-  const int G = gridDim.x / p.R;
-  const int x = blockIdx.x / p.R, y = blockIdx.x - x * p.R;
-  const int row0 = y * kBM;
-  CostPartition P;
-  P.init(bt, p.B, p.Hkv, G, kSegWeight);
-  const long long g_begin = P.begin(x), g_end = P.end(x);
-  // one reader per tile: evict it first; R row tiles read each tile R times
-  const bool one_reader = p.R == 1;
-
-  if (warp == kKProdWarp) {
-    // -------------------------------------------- producer: queries and keys
-    // The queries of segment s go in once S of segment s - 1 has read the
-    // previous ones; the keys run ahead independently, up to the ring depth.
-    if (lane == 0) {
-      const uint64_t pol_q = policy_evict_first();
-      const uint64_t pol_kv = one_reader ? policy_evict_first() : policy_evict_normal();
-      long long gk = g_begin, gq = g_begin;  // the next K tile's segment start, the next Q's segment
-      Segment sk;
-      int tk = 0;
-      if (gk < g_end) {
-        sk = locate(bt, P, p.B, gk, g_end);
-        tk = sk.t0;
-      }
-      int i = 0, qs = 0;  // K tiles and query tiles issued
-      uint64_t t_last = global_timer_ns();
-      int spins = 0, seen = 0;
-      while (gk < g_end || gq < g_end) {
-        bool progressed = false;
-        if (gq < g_end && mbar_test_wait(&bars[B_QEMPTY], (qs & 1) ^ 1)) {
-          const Segment sq = locate(bt, P, p.B, gq, g_end);
-          mbar_arrive_expect_tx(&bars[B_QFULL], C::kQBytes);
-          const int z = sq.b * p.n + row0 / p.group;  // the row tile's first node in [B n, H, D]
+  if (warp == kKProdWarp || warp == kVProdWarp) {
+    // ----------------------------------------------------------- producers
+    // Warp 8 the keys, warp 11 the values: one loop, so that its code is there
+    // once.  Lane 0 issues; the other lanes are there to clear the rows past a
+    // slab's last key in its last V tile.  One reader per tile: evict it first;
+    // R row tiles read each tile R times.
+    const bool keys = warp == kKProdWarp;
+    const uint64_t pol = p.R == 1 ? policy_evict_first() : policy_evict_normal();
+    const CUtensorMap* map = keys ? &tmK : &tmV;
+    unsigned char* ring = base + (keys ? C::off_K : off_V);
+    uint64_t* full = &bars[keys ? B_KFULL : B_VFULL];
+    uint64_t* empty = &bars[keys ? B_KEMPTY : B_VEMPTY];
+    const int depth = keys ? nk : nv;
+    int st = 0, issued = 0;
+    uint32_t phase = 1;  // the stage's parity as the waiter sees it
+    bool ok = true;
+    for (; s.any() && ok; s.next(bt, p.Hkv)) {
+      int row = (s.b * p.Hkv + s.h) * p.S_cap + s.t0 * kBN;
+      const int len = bt.len[s.b];
+      for (int t = s.t0; t < s.t1; ++t, row += kBN) {
+        ok = warp_wait_small(&empty[st], phase, abort_flag);
+        if (!ok) break;
+        unsigned char* dst = ring + st * C::kKV;
+        if (lane == 0) {
+          mbar_arrive_expect_tx(&full[st], C::kKV);
           for (int hd = 0; hd < C::kHalves; ++hd)
-            tc::tma_load_3d(base + C::off_Q + hd * kAtom, &tmQ, hd * 64, sq.h * p.group, z, &bars[B_QFULL], pol_q);
-          ++qs;
-          gq = sq.g_end;
-          progressed = true;
+            tc::tma_load_2d(dst + hd * kAtom, map, hd * 64, row, &full[st], pol);
         }
-        if (gk < g_end && mbar_test_wait(&bars[B_KEMPTY + i % nk], ((i / nk) & 1) ^ 1)) {
-          const int st = i % nk;
-          const int row = (sk.b * p.Hkv + sk.h) * p.S_cap + tk * kBN;
-          mbar_arrive_expect_tx(&bars[B_KFULL + st], C::kKV);
-          for (int hd = 0; hd < C::kHalves; ++hd)
-            tc::tma_load_2d(base + C::off_K + st * C::kKV + hd * kAtom, &tmK, hd * 64, row, &bars[B_KFULL + st],
-                            pol_kv);
-          ++i;
-          if (++tk == sk.t1) {
-            gk = sk.g_end;
-            if (gk < g_end) {
-              sk = locate(bt, P, p.B, gk, g_end);
-              tk = sk.t0;
-            }
-          }
-          progressed = true;
+        __syncwarp();
+        ++issued;
+        const int vrows = len - t * kBN;
+        if (!keys && vrows < kBN) {  // the slab's last tile: clear its V rows past the last key
+          ok = warp_wait_small(&full[st], phase ^ 1, abort_flag);
+          if (!ok) break;
+#pragma unroll 1
+          for (int idx = vrows * C::kHalves * 8 + lane; idx < kBN * C::kHalves * 8; idx += 32)
+            *reinterpret_cast<uint4*>(dst + ((idx >> 3) % C::kHalves) * kAtom + idx / (C::kHalves * 8) * 128 +
+                                      (idx & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
+          tc::fence_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bars[B_VCLR + st]);
         }
-        if (progressed) continue;
-        __nanosleep(32);
-        if (++spins < 32) continue;
-        spins = 0;  // every 32 idle polls: check for an abort or a stall of more than kWaitLimitNs
-        const uint64_t now = global_timer_ns();
-        if (i + qs != seen) {
-          seen = i + qs;
-          t_last = now;
+        if (++st == depth) {
+          st = 0;
+          phase ^= 1;
         }
-        if (*abort_flag) break;
-        if (now - t_last > kWaitLimitNs) {
-          *abort_flag = 1;
-          record_status(p.status, kStatusTimeout);
-          break;
-        }
-      }
-      if (gk < g_end || gq < g_end) {  // aborted: let issued loads land before the CTA exits
-        for (int j = (i > nk ? i - nk : 0); j < i; ++j) mbar_drain(&bars[B_KFULL + j % nk], (j / nk) & 1);
-        if (qs > 0) mbar_drain(&bars[B_QFULL], (qs - 1) & 1);
       }
     }
-  } else if (warp == kVProdWarp) {
-    // ------------------------------------------------------ producer: values
-    if (lane == 0) {
-      const uint64_t pol_kv = one_reader ? policy_evict_first() : policy_evict_normal();
-      int i = 0;
-      bool ok = true;
-      for (long long g = g_begin; g < g_end && ok;) {
-        const Segment sg = locate(bt, P, p.B, g, g_end);
-        const int row0k = (sg.b * p.Hkv + sg.h) * p.S_cap;
-        for (int t = sg.t0; t < sg.t1; ++t, ++i) {
-          const int st = i % nv;
-          if (!mbar_wait(&bars[B_VEMPTY + st], ((i / nv) & 1) ^ 1, abort_flag, p.status)) {
-            ok = false;
-            break;
-          }
-          mbar_arrive_expect_tx(&bars[B_VFULL + st], C::kKV);
-          for (int hd = 0; hd < C::kHalves; ++hd)
-            tc::tma_load_2d(base + off_V + st * C::kKV + hd * kAtom, &tmV, hd * 64, row0k + t * kBN,
-                            &bars[B_VFULL + st], pol_kv);
-        }
-        g = sg.g_end;
-      }
-      if (!ok)  // aborted: let issued loads land before the CTA exits
-        for (int j = (i > nv ? i - nv : 0); j < i; ++j) mbar_drain(&bars[B_VFULL + j % nv], (j / nv) & 1);
-    }
+    if (!ok && lane == 0)  // aborted: let issued loads land before the CTA exits
+      for (int j = (issued > depth ? issued - depth : 0); j < issued; ++j)
+        mbar_drain(&full[j % depth], (j / depth) & 1);
   } else if (warp == kSWarp || warp == kPVWarp) {
     // ----------------------------------------------------------- MMA issue
+    // Ring positions are counted, not divided out.
     if (lane == 0) {
-      const bool s_role = warp == kSWarp;
-      constexpr uint32_t idS = tc::idesc_bf16_f32(kBM, kBN, false, false);
-      constexpr uint32_t idO = tc::idesc_bf16_f32(kBM, D, false, true);
-      const uint64_t dQ = tc::sw128_desc(smem_u32(base + C::off_Q), 16, 1024);
-      const uint32_t sK = smem_u32(base + C::off_K), sV = smem_u32(base + off_V);
       bool ok = true;
-      int i = 0, seg = 0;
-      for (long long g = g_begin; g < g_end && ok; ++seg) {
-        const Segment s = locate(bt, P, p.B, g, g_end);
-        for (int t = s.t0; t < s.t1; ++t, ++i) {
-          const int bi = i % kSBufs;
-          if (s_role) {
-            // S(i) = Q K(i)^T into buffer i % 3, once P.V of tile i - 3 has read that buffer
-            if ((t == s.t0 && !mbar_wait(&bars[B_QFULL], seg & 1, abort_flag, p.status)) ||
-                !mbar_wait(&bars[B_KFULL + i % nk], (i / nk) & 1, abort_flag, p.status) ||
-                !mbar_wait(&bars[B_BFREE + bi], ((i / kSBufs) & 1) ^ 1, abort_flag, p.status)) {
-              ok = false;
-              break;
-            }
+      int bi = 0, st = 0, seg = 0;  // S buffer, ring stage, segment
+      uint32_t col = tmem, phase = 0;
+      if (warp == kSWarp) {
+        // S(i) = Q K(i)^T into buffer i % 3, once P.V of tile i - 3 has read
+        // that buffer; the segment's queries first, once S of the last segment
+        // has read the previous ones
+        constexpr uint32_t idS = tc::idesc_bf16_f32(kBM, kBN, false, false);
+        const uint64_t dQ = tc::sw128_desc(smem_u32(base + C::off_Q), 16, 1024);
+        const uint64_t dK0 = tc::sw128_desc(smem_u32(base + C::off_K), 16, 1024);
+        const uint64_t pol_q = policy_evict_first();
+        uint32_t b_phase = 1;
+        bool q_loading = false;
+        for (; s.any() && ok; s.next(bt, p.Hkv), ++seg) {
+          if (seg > 0) ok = mbar_wait_small(&bars[B_QEMPTY], (seg - 1) & 1, abort_flag);
+          if (!ok) break;
+          mbar_arrive_expect_tx(&bars[B_QFULL], C::kQBytes);
+          const int z = s.b * p.n + row0 / p.group;  // the row tile's first node in [B n, H, D]
+          for (int hd = 0; hd < C::kHalves; ++hd)
+            tc::tma_load_3d(base + C::off_Q + hd * kAtom, &tmQ, hd * 64, s.h * p.group, z, &bars[B_QFULL], pol_q);
+          q_loading = true;
+          ok = mbar_wait_small(&bars[B_QFULL], seg & 1, abort_flag);
+          if (ok) q_loading = false;
+#pragma unroll 1
+          for (int t = s.t1 - s.t0; ok && t > 0; --t) {
+            ok = mbar_wait_small(&bars[B_KFULL + st], phase, abort_flag) &&
+                 mbar_wait_small(&bars[B_BFREE + bi], b_phase, abort_flag);
+            if (!ok) break;
             tc::fence_after_sync();
-            const uint64_t dK = tc::sw128_desc(sK + (i % nk) * C::kKV, 16, 1024);
+            const uint64_t dK = dK0 + (uint64_t)st * desc_step(C::kKV);
 #pragma unroll
             for (int ks = 0; ks < D / 16; ++ks) {
               const uint64_t step = desc_step((ks >> 2) * kAtom + (ks & 3) * 32);
-              tc::mma_bf16(tmem + bi * kBN, dQ + step, dK + step, idS, ks > 0 ? 1u : 0u);
+              tc::mma_bf16(col, dQ + step, dK + step, idS, ks > 0 ? 1u : 0u);
             }
             tc::mma_commit(&bars[B_SFULL + bi]);
-            tc::mma_commit(&bars[B_KEMPTY + i % nk]);
-            if (t == s.t1 - 1) tc::mma_commit(&bars[B_QEMPTY]);
-          } else {
-            // O (+)= P_0(i) V_0(i) + P_1(i) V_1(i) over the key halves h = 0, 1: P_h in
-            // columns 64h .. 64h+31 of buffer i % 3; the segment's first tile starts O
-            if (!mbar_wait(&bars[B_PFULL + bi], (i / kSBufs) & 1, abort_flag, p.status) ||
-                !mbar_wait(&bars[B_VFULL + i % nv], (i / nv) & 1, abort_flag, p.status)) {
-              ok = false;
-              break;
+            tc::mma_commit(&bars[B_KEMPTY + st]);
+            if (t == 1) tc::mma_commit(&bars[B_QEMPTY]);
+            if (++st == nk) {
+              st = 0;
+              phase ^= 1;
             }
-            tc::fence_after_sync();
-            const uint64_t dV = tc::sw128_desc(sV + (i % nv) * C::kKV, kAtom, 1024);
-            const uint32_t pcol = tmem + bi * kBN;
-            tc::mma_bf16_ts(tmem + kTmemO, pcol, dV, idO, t == s.t0 ? 0u : 1u);
-#pragma unroll
-            for (int ks = 1; ks < kBN / 16; ++ks)
-              tc::mma_bf16_ts(tmem + kTmemO, pcol + (ks >> 2) * 64 + (ks & 3) * 8, dV + desc_step(ks * 16 * 128),
-                              idO, 1u);
-            tc::mma_commit(&bars[B_VEMPTY + i % nv]);
-            tc::mma_commit(&bars[B_ODONE + (i & 3)]);
-            tc::mma_commit(&bars[B_BFREE + bi]);
+            col += kBN;
+            if (++bi == kSBufs) {
+              bi = 0;
+              b_phase ^= 1;
+              col = tmem;
+            }
           }
         }
-        g = s.g_end;
+        if (q_loading) mbar_drain(&bars[B_QFULL], seg & 1);  // aborted: let the queries land
+        tc::mma_commit(&bars[B_MDONE]);  // every MMA finished before TMEM is released
+        mbar_drain(&bars[B_MDONE], 0);
+      } else {
+        // O (+)= P(i) V(i), P in the first 64 columns of buffer i % 3; the
+        // segment's first tile starts O, once its last value is read
+        constexpr uint32_t idO = tc::idesc_bf16_f32(kBM, D, false, true);
+        const uint64_t dV0 = tc::sw128_desc(smem_u32(base + off_V), kAtom, 1024);
+        uint32_t p_phase = 0, cleared = 0;  // cleared: bit s, parity of the clears of V stage s so far
+        int od = 0;
+        for (; s.any() && ok; s.next(bt, p.Hkv), ++seg) {
+          if (seg > 0) ok = mbar_wait_small(&bars[B_OFREE], (seg - 1) & 1, abort_flag);
+          const bool partial = s.t1 == bt.ntiles[s.b] && bt.len[s.b] < s.t1 * kBN;  // its last V tile gets cleared rows
+          uint32_t acc = 0;
+#pragma unroll 1
+          for (int t = s.t1 - s.t0; ok && t > 0; --t) {
+            ok = mbar_wait_small(&bars[B_VFULL + st], phase, abort_flag);
+            if (ok && t == 1 && partial) {
+              ok = mbar_wait_small(&bars[B_VCLR + st], (cleared >> st) & 1, abort_flag);
+              cleared ^= 1u << st;
+            }
+            ok = ok && mbar_wait_small(&bars[B_PFULL + bi], p_phase, abort_flag);
+            if (!ok) break;
+            tc::fence_after_sync();
+            const uint64_t dV = dV0 + (uint64_t)st * desc_step(C::kKV);
+#pragma unroll
+            for (int ks = 0; ks < kBN / 16; ++ks)
+              tc::mma_bf16_ts(tmem + kTmemO, col + ks * 8, dV + desc_step(ks * 16 * 128), idO, ks > 0 ? 1u : acc);
+            acc = 1;
+            tc::mma_commit(&bars[B_BFREE + bi]);
+            tc::mma_commit(&bars[B_VEMPTY + st]);
+            tc::mma_commit(&bars[B_ODONE + od]);
+            od = (od + 1) & 3;
+            if (++st == nv) {
+              st = 0;
+              phase ^= 1;
+            }
+            col += kBN;
+            if (++bi == kSBufs) {
+              bi = 0;
+              p_phase ^= 1;
+              col = tmem;
+            }
+          }
+        }
+        tc::mma_commit(&bars[B_MDONE + 1]);
+        mbar_drain(&bars[B_MDONE + 1], 0);
       }
-      const int role = s_role ? 0 : 1;
-      tc::mma_commit(&bars[B_MDONE + role]);  // every MMA finished before TMEM is released
-      mbar_drain(&bars[B_MDONE + role], 0);
     }
   } else {
     // ----------------------------------------------- softmax and epilogues
-    const int kh = warp >> 2, quarter = warp & 3;
+    const int grp = warp >> 2, quarter = warp & 3;  // this group's tiles: CTA-local index parity grp
     const int r = quarter * 32 + lane;  // this thread's row in the tile (its TMEM lane)
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-    const uint32_t o_col = kTmemO + kh * (D / 2);  // this group's half of the O columns
-    const int sid = threadIdx.x;                   // 0..255 among the softmax threads
     const float sl2 = p.scale_log2;
+    const uint64_t sc2 = f2(sl2, sl2);
     const int qrow = row0 + r;  // the slab's query row
     const bool valid = qrow < p.rows;
     const int node = valid ? qrow / p.group : 0;
@@ -353,10 +373,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     bool dead = false;
 
     // The share range of every slab split over several shares, for the merge
-    // kernel ((-1, -1): written out directly).
+    // kernel ((-1, -1): written out directly), and zeros for a prefix-only
+    // call's sequences without cached keys (an empty softmax).
     constexpr int kST = kSoftWarps * 32;
-    if (y == 0)
-      for (int bh = x * kST + sid; bh < p.B * p.Hkv; bh += G * kST) {
+    if (y == 0) {
+      CostPartition P;
+      P.init(bt, p.B, p.Hkv, G, kSegWeight);
+#pragma unroll 1
+      for (int bh = x * kST + (int)threadIdx.x; bh < p.B * p.Hkv; bh += G * kST) {
         const int b = bh / p.Hkv, nt = bt.ntiles[b];
         int2 rg = make_int2(-1, -1);
         if (nt > 0) {
@@ -366,179 +390,173 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         p.ranges[bh] = rg;
       }
-    if (!p.tree) {  // prefix only: a sequence without cached keys gets zeros (an empty softmax)
-      const long long total = (long long)p.B * p.n * p.H * D;
-      for (long long idx = (long long)blockIdx.x * kST + sid; idx < total; idx += (long long)gridDim.x * kST)
-        if (bt.ntiles[idx / ((long long)p.n * p.H * D)] == 0) p.out[idx] = 0.f;
     }
+    if (!p.tree)
+      zero_empty(bt, p.B, (long long)p.n * p.H * D, p.out, (int)blockIdx.x * kST + (int)threadIdx.x,
+                 (int)gridDim.x * kST);
 
-    int i = 0;  // CTA-local key tile
-    for (long long g = g_begin; g < g_end;) {
-      const Segment s = locate(bt, P, p.B, g, g_end);
-      const int plen = bt.plen[s.b], len = bt.len[s.b];
+    unsigned i = 0;  // CTA-local index of the segment's first tile
+    for (; s.any(); s.next(bt, p.Hkv)) {
+      const int plen = bt.plen[s.b], nt = s.t1 - s.t0;
+      const unsigned jl = i + nt - 1;  // the segment's last tile
       // this row's node's ancestor-or-self set, found at the first tile that
-      // reaches the tree keys
+      // reaches the tree keys (prefix only: no tree keys)
       uint64_t anc = 0;
-      bool anc_ready = false;
-      float m_used = -CUDART_INF_F, l = 0.f;  // l: this key half's share of the row sum
-      for (int t = s.t0; t < s.t1; ++t, ++i) {
-        const int bi = i % kSBufs;
-        uint32_t sv[64];
-        if (!dead) dead = !warp_wait(&bars[B_SFULL + bi], (i / kSBufs) & 1, abort_flag, p.status);
-        if (!dead) {
-          tc::fence_after_sync();
-          tc::tmem_ld32(lane_base + bi * kBN + kh * 64, *reinterpret_cast<uint32_t(*)[32]>(sv));
-          tc::tmem_ld32(lane_base + bi * kBN + kh * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(sv + 32));
-          tc::tmem_wait_ld();
-        } else {
-#pragma unroll
-          for (int e = 0; e < 64; ++e) sv[e] = 0u;
-        }
-        // keys of this half from k0: the prefix is visible, tree key c only to
-        // the rows of c's descendants-or-self, and nothing past the tree
-        const int k0 = t * kBN + kh * 64;
-        if (k0 + 64 > plen) {  // warp-uniform
-          if (p.tree && !anc_ready) {
+      bool anc_ready = !p.tree;
+      float m_own = -CUDART_INF_F, l = 0.f;  // the sum over this group's tiles and the reference it is taken against
+      for (int t = (int)((i ^ grp) & 1u); t < nt; t += 2) {
+        const unsigned j = i + t, bi = j % kSBufs;
+        const uint32_t s_col = lane_base + bi * kBN;
+        if (!opaque(dead)) dead = !warp_wait_small(&bars[B_SFULL + bi], (j / kSBufs) & 1, abort_flag);
+        tc::fence_after_sync();
+        // keys this row does not see (tree keys that are no ancestors, and what
+        // lies past the tree): -inf, written back to the S buffer
+        const int k0 = (s.t0 + t) * kBN - plen;  // the tile's first key, past the prefix
+        if (k0 + kBN > 0) {
+          if (!opaque(anc_ready)) {
             anc = ancestors(p.parent + (size_t)s.b * p.n, p.n, node, valid, lane);
             anc_ready = true;
           }
+#pragma unroll 1
+          for (int c = 0; c < opaque(kBN / 32); ++c) {
+            uint32_t o[32];
+            tc::tmem_ld32(s_col + c * 32, o);
+            tc::tmem_wait_ld();
+            const uint32_t vis = (uint32_t)visible_keys(anc, k0 + c * 32);
 #pragma unroll
-          for (int e = 0; e < 64; ++e) {
-            const int kk = k0 + e;
-            const bool vis = kk < plen || (kk < len && ((anc >> ((kk - plen) & 63)) & 1ull));
-            sv[e] = vis ? sv[e] : 0xff800000u;
+            for (int e = 0; e < 32; ++e) o[e] = (vis & (1u << e)) ? o[e] : 0xff800000u;
+            tc::tmem_st32(s_col + c * 32, o);
           }
-        }
-        float mx[4] = {__uint_as_float(sv[0]), __uint_as_float(sv[1]), __uint_as_float(sv[2]),
-                       __uint_as_float(sv[3])};
-#pragma unroll
-        for (int e = 4; e < 64; e += 8) {
-          mx[0] = fmax3(mx[0], __uint_as_float(sv[e]), __uint_as_float(sv[e + 1]));
-          mx[1] = fmax3(mx[1], __uint_as_float(sv[e + 2]), __uint_as_float(sv[e + 3]));
-          if (e + 4 < 64) {
-            mx[2] = fmax3(mx[2], __uint_as_float(sv[e + 4]), __uint_as_float(sv[e + 5]));
-            mx[3] = fmax3(mx[3], __uint_as_float(sv[e + 6]), __uint_as_float(sv[e + 7]));
-          }
-        }
-        float tmax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sl2;
-        // the row max over both key halves: through column 63 of each half,
-        // already read; the pair barrier orders the partner's read after the write
-        if (!dead) {
-          tc::tmem_st1(lane_base + bi * kBN + kh * 64 + 63, __float_as_uint(tmax));
           tc::tmem_wait_st();
         }
-        tc::fence_before_sync();
-        pair_sync(quarter);
-        if (!dead) {
-          tc::fence_after_sync();
-          const uint32_t o = tc::tmem_ld1(lane_base + bi * kBN + (kh ^ 1) * 64 + 63);
-          tc::tmem_wait_ld();
-          tmax = fmaxf(tmax, __uint_as_float(o));
-        }
-        const bool need = tmax > m_used + kRescaleLog2;
-        if (__any_sync(0xffffffffu, need)) {
-          const float m_new = need ? tmax : m_used;
-          const float f = need ? fast_exp2(m_used - m_new) : 1.f;
-          l *= f;
-          if (t > s.t0 && !dead) {  // O holds the P.V of this segment's earlier tiles: rescale this group's half
-            dead = !warp_wait(&bars[B_ODONE + ((i - 1) & 3)], ((i - 1) >> 2) & 1, abort_flag, p.status);
-            if (!dead) {
-              tc::fence_after_sync();
+        // The scores are read from TMEM twice, 64 at a time in rolled loops
+        // (row max, then exponentials): unrolled over a whole 128-key row the
+        // loop body outgrows the instruction cache.
+        float mx[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
 #pragma unroll 1
-              for (int c = 0; c < D / 64; ++c) {
-                uint32_t o[32];
-                tc::tmem_ld32(lane_base + o_col + c * 32, o);
-                tc::tmem_wait_ld();
+        for (int hf = 0; hf < opaque(2); ++hf) {
+          uint32_t sv[64];
+          tc::tmem_ld32(s_col + hf * 64, *reinterpret_cast<uint32_t(*)[32]>(sv));
+          tc::tmem_ld32(s_col + hf * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(sv + 32));
+          tc::tmem_wait_ld();
 #pragma unroll
-                for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * f);
-                tc::tmem_st32(lane_base + o_col + c * 32, o);
-              }
-              tc::tmem_wait_st();
-            }
+          for (int e = 0; e < 64; e += 8)
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              mx[q] = fmax3(mx[q], __uint_as_float(sv[e + 2 * q]), __uint_as_float(sv[e + 2 * q + 1]));
+        }
+        const float tmax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sl2;
+        // The reference max passes from tile to tile, so from group to group
+        // (one slot: a thread reads its row's before it writes the next).
+        float m_prev = -CUDART_INF_F;
+        if (t > 0) {
+          turn_wait(quarter, j - 1);
+          m_prev = rowbuf[r];
+        }
+        const bool need = tmax > m_prev + kRescaleLog2;
+        const float m_used = need ? tmax : m_prev;
+        rowbuf[r] = m_used;
+        turn_pass(quarter, j);
+        if (__any_sync(0xffffffffu, need) && t > 0 && !dead) {
+          // O holds the P.V of this segment's earlier tiles, the other group's last one included: rescale it
+          dead = !warp_wait_small(&bars[B_ODONE + ((j - 1) & 3)], ((j - 1) >> 2) & 1, abort_flag);
+          const float f = need ? fast_exp2(m_prev - m_used) : 1.f;
+          tc::fence_after_sync();
+#pragma unroll 1
+          for (int c = 0; c < opaque(D / 32); ++c) {
+            uint32_t o[32];
+            tc::tmem_ld32(lane_base + kTmemO + c * 32, o);
+            tc::tmem_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * f);
+            tc::tmem_st32(lane_base + kTmemO + c * 32, o);
           }
-          m_used = m_new;
+          tc::tmem_wait_st();
+        }
+        if (m_own != m_used) {
+          l *= fast_exp2(m_own - m_used);  // 0 while there is no sum
+          m_own = m_used;
         }
         const float m_eff = m_used == -CUDART_INF_F ? 0.f : m_used;
-        const uint64_t sc2 = f2(sl2, sl2), nm2 = f2(-m_eff, -m_eff);
+        const uint64_t nm2 = f2(-m_eff, -m_eff);
         uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
-        uint32_t pk[32];
+#pragma unroll 1
+        for (int hf = 0; hf < opaque(2); ++hf) {
+          uint32_t sv[64], pk[32];
+          tc::tmem_ld32(s_col + hf * 64, *reinterpret_cast<uint32_t(*)[32]>(sv));
+          tc::tmem_ld32(s_col + hf * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(sv + 32));
+          tc::tmem_wait_ld();
 #pragma unroll
-        for (int e = 0; e < 32; ++e) {
-          float x0, x1;
-          unf2(ffma2(f2(__uint_as_float(sv[2 * e]), __uint_as_float(sv[2 * e + 1])), sc2, nm2), x0, x1);
-          const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
-          acc[e & 3] = fadd2(acc[e & 3], f2(p0, p1));
-          pk[e] = pack_bf16x2(p0, p1);
+          for (int e = 0; e < 32; ++e) {
+            float x0, x1;
+            unf2(ffma2(f2(__uint_as_float(sv[2 * e]), __uint_as_float(sv[2 * e + 1])), sc2, nm2), x0, x1);
+            const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
+            acc[e & 3] = fadd2(acc[e & 3], f2(p0, p1));
+            pk[e] = pack_bf16x2(p0, p1);
+          }
+          tc::tmem_st32(s_col + hf * 32, pk);  // over scores already read
         }
-        {
-          float a0, a1, b0, b1;
-          unf2(fadd2(acc[0], acc[1]), a0, a1);
-          unf2(fadd2(acc[2], acc[3]), b0, b1);
-          l += (a0 + a1) + (b0 + b1);
-        }
-        if (!dead) {  // P over the first 32 columns of this half's part of the S buffer
-          tc::tmem_st32(lane_base + bi * kBN + kh * 64, pk);
-          tc::tmem_wait_st();
-        }
-        const int vrows = len - t * kBN;
-        if (vrows < kBN) {  // the slab's last tile: clear V rows past its last key
-          const int st = i % nv;
-          if (!dead) dead = !warp_wait(&bars[B_VFULL + st], (i / nv) & 1, abort_flag, p.status);
-          if (!dead)
-            for (int idx = sid; idx < (kBN - vrows) * C::kHalves * 8; idx += kST) {
-              const int row = vrows + idx / (C::kHalves * 8), rem = idx % (C::kHalves * 8);
-              *reinterpret_cast<uint4*>(base + off_V + st * C::kKV + (rem >> 3) * kAtom + row * 128 + (rem & 7) * 16) =
-                  make_uint4(0u, 0u, 0u, 0u);
-            }
-          tc::fence_async_smem();
-        }
+        tc::tmem_wait_st();
         tc::fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars[B_PFULL + bi]);
+        float a0, a1, b0, b1;
+        unf2(fadd2(acc[0], acc[1]), a0, a1);
+        unf2(fadd2(acc[2], acc[3]), b0, b1);
+        l += (a0 + a1) + (b0 + b1);
       }
 
-      // ---- segment epilogue: the row sum over both halves, then each group
-      // writes its half of the head dims, O / l or a split partial.  The next
-      // segment's first P.V (which starts O afresh) waits for this group's
-      // P of that tile, so O is read here before it is overwritten.
-      lsum[kh * kBM + r] = l;
+      // ---- segment epilogue: the row sum over both groups, then each writes
+      // its half of the head dims, O / l or a split partial.  The group that did
+      // not do the last tile takes its sum to that tile's reference first, and
+      // leaves it where the reference was.
+      const bool mine = ((jl ^ grp) & 1u) == 0;
+      if (!mine) {
+        turn_wait(quarter, jl);
+        const float m_last = rowbuf[r];
+        if (m_own != m_last) l *= fast_exp2(m_own - m_last);
+        m_own = m_last;
+      }
+      rowbuf[(mine ? kBM : 0) + r] = l;
       pair_sync(quarter);
-      const float L = lsum[r] + lsum[kBM + r];
-      const int jl = i - 1;  // the segment's last tile
-      if (!dead) dead = !warp_wait(&bars[B_ODONE + (jl & 3)], (jl >> 2) & 1, abort_flag, p.status);
-      if (!dead) {
-        tc::fence_after_sync();
-        uint32_t o[D / 2];
+      const float L = rowbuf[r] + rowbuf[kBM + r];
+      pair_sync(quarter);  // read, before the next segment's reference goes in
+      if (!dead) dead = !warp_wait_small(&bars[B_ODONE + (jl & 3)], (jl >> 2) & 1, abort_flag);
+      tc::fence_after_sync();
+      uint32_t o[D / 2];
 #pragma unroll
-        for (int c = 0; c < D / 64; ++c)
-          tc::tmem_ld32(lane_base + o_col + c * 32, *reinterpret_cast<uint32_t(*)[32]>(o + 32 * c));
-        tc::tmem_wait_ld();
-        if (valid) {
-          if (s.c_first == s.c_last) {  // the whole slab in this share: the output row
-            const float inv = L > 0.f ? 1.f / L : 0.f;
-            float* dst = p.out + om.row(s.b, s.h, qrow, p.rows) * D + kh * (D / 2);
+      for (int c = 0; c < D / 64; ++c)
+        tc::tmem_ld32(lane_base + kTmemO + grp * (D / 2) + c * 32, *reinterpret_cast<uint32_t(*)[32]>(o + 32 * c));
+      tc::tmem_wait_ld();
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars[B_OFREE]);
+      if (valid && !dead) {
+        if (s.whole(bt)) {  // the whole slab in this share: the output row
+          const float inv = L > 0.f ? 1.f / L : 0.f;
+          float* dst = p.out + om.row(s.b, s.h, qrow, p.rows) * D + grp * (D / 2);
 #pragma unroll
-            for (int e = 0; e < D / 2; e += 4)
-              *reinterpret_cast<float4*>(dst + e) =
-                  make_float4(__uint_as_float(o[e]) * inv, __uint_as_float(o[e + 1]) * inv,
-                              __uint_as_float(o[e + 2]) * inv, __uint_as_float(o[e + 3]) * inv);
-          } else {  // the share's partial [max, sum, o] (a partial row is 8-byte aligned)
-            float* dst = partial_slot(p.partials, x + s.b * p.Hkv + s.h, p.rows, D) + (size_t)qrow * (D + 2);
-            if (kh == 0) *reinterpret_cast<float2*>(dst) = make_float2(m_used, L);
+          for (int e = 0; e < D / 2; e += 4)
+            *reinterpret_cast<float4*>(dst + e) =
+                make_float4(__uint_as_float(o[e]) * inv, __uint_as_float(o[e + 1]) * inv,
+                            __uint_as_float(o[e + 2]) * inv, __uint_as_float(o[e + 3]) * inv);
+        } else {  // the share's partial [max, sum, o] (a partial row is 8-byte aligned)
+          float* dst = partial_slot(p.partials, x + s.b * p.Hkv + s.h, p.rows, D) + (size_t)qrow * (D + 2);
+          if (grp == 0) *reinterpret_cast<float2*>(dst) = make_float2(m_own, L);
 #pragma unroll
-            for (int e = 0; e < D / 2; e += 2)
-              *reinterpret_cast<float2*>(dst + 2 + kh * (D / 2) + e) =
-                  make_float2(__uint_as_float(o[e]), __uint_as_float(o[e + 1]));
-          }
+          for (int e = 0; e < D / 2; e += 2)
+            *reinterpret_cast<float2*>(dst + 2 + grp * (D / 2) + e) =
+                make_float2(__uint_as_float(o[e]), __uint_as_float(o[e + 1]));
         }
       }
-      g = s.g_end;
+      i += nt;
     }
   }
 
-  __syncwarp();  // the producer and MMA warps reconverge after their single-lane loops
+  __syncwarp();  // the MMA warps reconverge after their single-lane loops
   tc::fence_before_sync();
   __syncthreads();
+  if (threadIdx.x == 0) record_abort(abort_flag, p.status);
   if (warp == kSWarp) {
     tc::fence_after_sync();
     tc::tmem_dealloc(tmem, kTmemCols);
