@@ -125,7 +125,11 @@ glide_status glide_cross_attn(const glide_attn_desc* desc, const void* q_draft, 
   if (workspace_bytes < attn_ws_bytes(desc, 1)) return GLIDE_ERR_INVALID;
   glide::AttnArgs a = make_args(desc, q_draft, K_cache, V_cache, kv_len, nullptr, out, workspace, 1, max_kv_len);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (a.Hkv == a.H) return from_cuda(glide::launch_cross_attn(a, st));
+  if (a.Hkv == a.H) {
+    cudaError_t e = glide::launch_cross_direct(a, st);
+    if (e != cudaErrorNotSupported) return from_cuda(e);
+    return from_cuda(glide::launch_cross_attn(a, st));
+  }
   // Grouped-query attention: a cached head serves H / H_kv draft queries, so
   // one pass over its keys is a small dense contraction -- the verification
   // kernels without tree keys, with the group's queries as their rows.

@@ -1,0 +1,281 @@
+// GliDe cross-attention (Section 3.1): one draft query per (sequence, head)
+// attends to every cached key, straight from global memory to registers.
+//
+// What bounds it.  The step reads every K and V byte once at ~1 flop per byte,
+// so HBM bounds long caches and the fixed parts of a call bound short ones (a
+// single user's decode: 32 heads, 2048 keys, 33 MB, 5 us of bytes).  The
+// streaming kernel of cross_attn.cu spends ~7 us beside the bytes on a chunk
+// table, run-time claims, shared-memory rings and a second kernel for the split
+// merge.  Here a call is one kernel with little to start up:
+// * a cluster of C CTAs serves one (b, h); its 8 C warps take the 16-key tiles
+//   in turn.  A warp loads a tile's 8 KB into registers, the next keys while it
+//   works on this tile's values; two CTAs an SM keep ~200 KB an SM in flight
+//   without barriers or rings;
+// * the warps' partial softmax results meet in shared memory, the C CTAs' in
+//   distributed shared memory, so nothing passes through global memory and the
+//   workspace is not used.  The order of all sums is fixed: repeated calls are
+//   bit-identical;
+// * the hardware hands the clusters to the SMs as they free up, which evens out
+//   what the SMs are served as well as the claims did.
+// Measured back to back over three caches in turn, streaming kernel -> this one
+// (us): 32 heads, 2048 keys 11.8 -> 7.8; 128 keys 6.9 -> 3.7; 4 x 32 heads,
+// 4096 keys 47.1 -> 40.9; ragged 32.8 -> 29.3; 4 x 52 heads, 16384 keys
+// 249.8 -> 239.3 (7.3 TB/s), ragged 157.9 -> 154.1; D = 64, 4 x 32 heads,
+// 2048 keys 25.2 -> 13.5.
+#include <cuda_bf16.h>
+#include <math_constants.h>
+
+#include "attn_common.cuh"
+#include "common.cuh"
+#include "kernels.h"
+
+namespace glide {
+namespace {
+
+constexpr int kTK = 16;       // keys per tile
+constexpr int kWarps = 8;     // warps per CTA
+constexpr int kThreads = kWarps * 32;
+constexpr int kMaxCluster = 8;
+
+struct DirectParams {
+  const void* q;
+  const void* K;
+  const void* V;
+  const int* kv_len;
+  float* out;
+  int H, S_cap, max_kv_len;
+  int C;  // CTAs of a cluster
+  float scale_log2;
+};
+
+// 16 bytes that are used once: past L1 (a programmatic launch may find old
+// lines there) and first to leave L2.
+__device__ __forceinline__ uint4 load_once(const void* p, uint64_t policy) {
+  uint4 v;
+  asm volatile("ld.global.cg.L2::cache_hint.v4.b32 {%0, %1, %2, %3}, [%4], %5;"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p), "l"(policy));
+  return v;
+}
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// A float of CTA `rank` of this cluster, at the address it has in this CTA.
+__device__ __forceinline__ float load_peer(const float* p, uint32_t rank) {
+  uint32_t a;
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+
+template <typename T, int D>
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 2 : 1) cross_direct_kernel(const DirectParams p) {
+  using G = GroupMap<T, D>;
+  __shared__ float red[kWarps][D];
+  __shared__ float2 stat[kWarps];
+  __shared__ float part[D + 2];  // this CTA's (max, sum, o) for its peers
+  pdl_wait();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = (int)cluster_rank();
+  const int bh = blockIdx.x / p.C, b = bh / p.H;
+  int n = p.kv_len[b];
+  n = n < 0 ? 0 : (n > p.max_kv_len ? p.max_kv_len : n);
+  const int sub = lane & 7, g4 = (lane >> 3) * 4;  // lane group g takes keys 4g..4g+3 of each tile
+  const float sl2 = p.scale_log2;
+  const uint64_t pol = policy_evict_first();
+  const size_t slab = (size_t)bh * p.S_cap * D * sizeof(T);
+  const unsigned char* Kg = static_cast<const unsigned char*>(p.K) + slab;
+  const unsigned char* Vg = static_cast<const unsigned char*>(p.V) + slab;
+  uint4 qc[G::kNC];
+  {
+    const unsigned char* qrow = static_cast<const unsigned char*>(p.q) + (size_t)bh * G::kRowBytes;
+#pragma unroll
+    for (int m = 0; m < G::kNC; ++m) qc[m] = __ldcg(reinterpret_cast<const uint4*>(qrow + (sub + 8 * m) * 16));
+  }
+  float m = -CUDART_INF_F, l = 0.f;
+  uint64_t o2[G::kPairs];
+#pragma unroll
+  for (int e = 0; e < G::kPairs; ++e) o2[e] = 0ull;
+
+  // this lane's chunks of the group's four rows of a tile; rows past the end
+  // (the cache may hold anything there, or end) are zeros
+  auto load = [&](uint4 (&r)[4][G::kNC], const unsigned char* base, int key0) {
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+      for (int c = 0; c < G::kNC; ++c) {
+        r[kk][c] = make_uint4(0u, 0u, 0u, 0u);
+        if (key0 + g4 + kk < n)
+          r[kk][c] = load_once(base + (size_t)(key0 + g4 + kk) * G::kRowBytes + (sub + 8 * c) * 16, pol);
+      }
+  };
+  const int step = p.C * kWarps * kTK;
+  int key0 = (rank * kWarps + warp) * kTK;
+  uint4 kr[4][G::kNC], vr[4][G::kNC];
+  load(kr, Kg, key0);
+#pragma unroll 1
+  for (; key0 < n; key0 += step) {
+    load(vr, Vg, key0);
+    // partial scores of this group's 4 keys over this lane's dims
+    float s4[4];
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) {
+      float acc[2] = {0.f, 0.f};
+#pragma unroll
+      for (int c = 0; c < G::kNC; ++c) dot_chunk<T>(qc[c], kr[kk][c], acc);
+      s4[kk] = acc[0] + acc[1];
+    }
+    load(kr, Kg, key0 + step);  // the next tile's keys, under this one's softmax and values
+    float sc = group8_reduce4(s4, lane) * sl2;  // score of key lane / 2 of the tile
+    if (key0 + (lane >> 1) >= n) sc = -CUDART_INF_F;
+    const float m_new = fmaxf(m, warp_max(sc));
+    const float corr = fast_exp2(m - m_new);
+    const float pe = fast_exp2(sc - m_new);
+    l = l * corr + ((lane & 1) ? 0.f : pe);  // each key is held by two lanes: count it once
+    const uint64_t corr2 = f2pack(corr, corr);
+#pragma unroll
+    for (int e = 0; e < G::kPairs; ++e) o2[e] = f2mul(o2[e], corr2);
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) {
+      const float pk = __shfl_sync(0xffffffffu, pe, (lane & ~7) + 2 * kk);
+      const uint64_t p2 = f2pack(pk, pk);
+#pragma unroll
+      for (int c = 0; c < G::kNC; ++c) axpy_chunk<T>(p2, vr[kk][c], o2 + c * G::kPairsPerChunk);
+    }
+    m = m_new;
+  }
+
+  // the warp's result: lane groups merged, lanes 0-7 hold o
+  l = warp_sum(l);
+#pragma unroll
+  for (int e = 0; e < G::kPairs; ++e) {
+    float2 v = f2unpack(o2[e]);
+    v.x += __shfl_xor_sync(0xffffffffu, v.x, 8);
+    v.y += __shfl_xor_sync(0xffffffffu, v.y, 8);
+    v.x += __shfl_xor_sync(0xffffffffu, v.x, 16);
+    v.y += __shfl_xor_sync(0xffffffffu, v.y, 16);
+    const int d = (sub + 8 * (e / G::kPairsPerChunk)) * G::kChunkElems + 2 * (e % G::kPairsPerChunk);
+    if (lane < 8) *reinterpret_cast<float2*>(&red[warp][d]) = v;
+  }
+  if (lane == 0) stat[warp] = make_float2(m, l);
+  __syncthreads();
+  // the CTA's: a warp without a tile has max -inf and weight 0
+  if (threadIdx.x < D) {
+    float M = -CUDART_INF_F, L = 0.f, O = 0.f;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) M = fmaxf(M, stat[w].x);
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      const float f = stat[w].x == -CUDART_INF_F ? 0.f : fast_exp2(stat[w].x - M);
+      L += f * stat[w].y;
+      O += f * red[w][threadIdx.x];
+    }
+    part[2 + threadIdx.x] = O;
+    if (threadIdx.x == 0) {
+      part[0] = M;
+      part[1] = L;
+    }
+  }
+  cluster_arrive();
+  cluster_wait();
+  // the cluster's: CTA r writes dims r D / C ..
+  const int dims = D / p.C;
+  if (threadIdx.x < dims) {
+    const int d = rank * dims + threadIdx.x;
+    float M = -CUDART_INF_F, L = 0.f, O = 0.f;
+    float pm[kMaxCluster], pl[kMaxCluster], po[kMaxCluster];
+#pragma unroll
+    for (int c = 0; c < kMaxCluster; ++c) {
+      const uint32_t peer = c < p.C ? c : 0;
+      pm[c] = c < p.C ? load_peer(&part[0], peer) : -CUDART_INF_F;
+      pl[c] = load_peer(&part[1], peer);
+      po[c] = load_peer(&part[2 + d], peer);
+      M = fmaxf(M, pm[c]);
+    }
+#pragma unroll
+    for (int c = 0; c < kMaxCluster; ++c) {
+      const float f = pm[c] == -CUDART_INF_F ? 0.f : fast_exp2(pm[c] - M);
+      L += f * pl[c];
+      O += f * po[c];
+    }
+    p.out[(size_t)bh * D + d] = L > 0.f ? O / L : 0.f;  // no cached keys: an empty softmax, zero
+  }
+  cluster_arrive();  // a CTA's shared memory stays until its peers have read it
+  cluster_wait();
+}
+
+template <typename T, int D>
+cudaError_t launch_typed(const AttnArgs& a, int C, cudaStream_t st) {
+  DirectParams p;
+  p.q = a.q; p.K = a.K; p.V = a.V; p.kv_len = a.kv_len; p.out = a.out;
+  p.H = a.H; p.S_cap = a.S_cap; p.max_kv_len = a.max_kv_len;
+  p.C = C;
+  p.scale_log2 = a.scale * kLog2e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(a.B * a.H * C));
+  cfg.blockDim = dim3(kThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)C;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, cross_direct_kernel<T, D>, p);
+}
+
+}  // namespace
+
+cudaError_t launch_cross_direct(const AttnArgs& a, cudaStream_t st) {
+  const long long BH = (long long)a.B * a.H;
+  const int per_sm = a.dtype == 0 ? 2 : 1;
+  const long long slots = (long long)per_sm * sm_count();
+  auto rounds = [&](int C) { return (a.max_kv_len + C * kWarps * kTK - 1) / (C * kWarps * kTK); };  // tiles per warp
+  // How full the waves of BH * C CTAs are.
+  auto fill = [&](int C) {
+    const double waves = (double)(BH * C) / (double)slots;
+    return waves / (double)((BH * C + slots - 1) / slots);
+  };
+  // CTAs per (b, h): as many as one wave holds (each wave costs its start, ~3
+  // us: 2 x 32 heads, 512 keys, C = 4 and 8: 4.7 and 7.9 us), but no more than
+  // there are tiles.
+  int C = kMaxCluster;
+  while (C > 1 && (BH * C > slots || C * kWarps * kTK >= 2 * a.max_kv_len)) C >>= 1;
+  // Long caches: shorter CTAs in more waves, so that the SMs end together (4 x
+  // 52 heads, 16384 keys, C = 1 and 4: 243.2 and 239.3 us, ragged 172.7 and
+  // 154.1).  More than a wave of (b, h) needs it sooner, and where one CTA each
+  // leaves a thin last wave, two fill it (8 x 40 heads, 2048 keys, C = 1 and 2:
+  // 65.0 and 59.9 us; 16 x 32 heads, whose waves are as full with one: 79.7
+  // and 85.0).
+  if (rounds(C) >= (BH > slots ? 32 : 64)) {
+    if (C < 4) C = 4;
+  } else if (BH > slots && rounds(C) >= 16 && fill(2) > fill(1) + 0.05) {
+    C = 2;
+  }
+  // A few (b, h) with long caches do not fill the SMs even at C = 8: the
+  // streaming kernel spreads them over all (8 heads, 8192 and 16384 keys, here
+  // 11.6 and 20.4 us, there 13.0 and 20.4; below that here is faster, above
+  // and for fewer heads there).  It also honours a bound on the CTAs.
+  if (BH < 12 && a.max_kv_len > 8192) return cudaErrorNotSupported;
+  // The same where fp32's one CTA an SM leaves clusters of 8 without room in
+  // the GPCs (16 heads, 4096 keys: here 18.9 us, there 16.3).
+  if (a.dtype != 0 && C == kMaxCluster && BH > 8 && a.max_kv_len > 2048) return cudaErrorNotSupported;
+  if (a.max_ctas > 0 && BH * C > a.max_ctas) return cudaErrorNotSupported;
+  if (BH * C > 0x7fffffffLL) return cudaErrorNotSupported;  // grid
+  if (a.dtype == 0 && a.D == 128) return launch_typed<__nv_bfloat16, 128>(a, C, st);
+  if (a.dtype == 0 && a.D == 64) return launch_typed<__nv_bfloat16, 64>(a, C, st);
+  if (a.dtype == 1 && a.D == 128) return launch_typed<float, 128>(a, C, st);
+  if (a.dtype == 1 && a.D == 64) return launch_typed<float, 64>(a, C, st);
+  return cudaErrorNotSupported;
+}
+
+}  // namespace glide
