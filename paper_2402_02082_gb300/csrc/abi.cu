@@ -142,6 +142,8 @@ glide_status glide_cross_attn(const glide_attn_desc* desc, const void* q_draft, 
     cudaError_t e = glide::launch_tree_attn_tc(a, st);
     if (e != cudaErrorNotSupported) return from_cuda(e);
   }
+  cudaError_t e = glide::launch_tree_direct(a, st);
+  if (e != cudaErrorNotSupported) return from_cuda(e);
   return from_cuda(glide::launch_tree_attn_fma(a, st));
 }
 
@@ -168,6 +170,8 @@ glide_status tree_verify_attn(const glide_attn_desc* desc, const void* q_tree, i
     cudaError_t e = glide::launch_tree_attn_tc(a, st);
     if (e != cudaErrorNotSupported) return from_cuda(e);
   }
+  cudaError_t e = glide::launch_tree_direct(a, st);
+  if (e != cudaErrorNotSupported) return from_cuda(e);
   return from_cuda(glide::launch_tree_attn_fma(a, st));
 }
 

@@ -48,32 +48,6 @@ struct DirectParams {
   float scale_log2;
 };
 
-// 16 bytes that are used once: past L1 (a programmatic launch may find old
-// lines there) and first to leave L2.
-__device__ __forceinline__ uint4 load_once(const void* p, uint64_t policy) {
-  uint4 v;
-  asm volatile("ld.global.cg.L2::cache_hint.v4.b32 {%0, %1, %2, %3}, [%4], %5;"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(p), "l"(policy));
-  return v;
-}
-
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-// A float of CTA `rank` of this cluster, at the address it has in this CTA.
-__device__ __forceinline__ float load_peer(const float* p, uint32_t rank) {
-  uint32_t a;
-  float v;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
-  return v;
-}
-
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 2 : 1) cross_direct_kernel(const DirectParams p) {
   using G = GroupMap<T, D>;
@@ -135,8 +109,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 2 : 1) cross_direct
     float sc = group8_reduce4(s4, lane) * sl2;  // score of key lane / 2 of the tile
     if (key0 + (lane >> 1) >= n) sc = -CUDART_INF_F;
     const float m_new = fmaxf(m, warp_max(sc));
-    const float corr = fast_exp2(m - m_new);
-    const float pe = fast_exp2(sc - m_new);
+    const float ref = m_new == -CUDART_INF_F ? 0.f : m_new;  // scores of -inf weigh 0; a NaN stays one
+    const float corr = fast_exp2(m - ref);
+    const float pe = fast_exp2(sc - ref);
     l = l * corr + ((lane & 1) ? 0.f : pe);  // each key is held by two lanes: count it once
     const uint64_t corr2 = f2pack(corr, corr);
 #pragma unroll
@@ -165,14 +140,15 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 2 : 1) cross_direct
   }
   if (lane == 0) stat[warp] = make_float2(m, l);
   __syncthreads();
-  // the CTA's: a warp without a tile has max -inf and weight 0
+  // the CTA's: a warp without a tile has max -inf, weight 0 and zeros
   if (threadIdx.x < D) {
     float M = -CUDART_INF_F, L = 0.f, O = 0.f;
 #pragma unroll
     for (int w = 0; w < kWarps; ++w) M = fmaxf(M, stat[w].x);
+    const float ref = M == -CUDART_INF_F ? 0.f : M;
 #pragma unroll
     for (int w = 0; w < kWarps; ++w) {
-      const float f = stat[w].x == -CUDART_INF_F ? 0.f : fast_exp2(stat[w].x - M);
+      const float f = fast_exp2(stat[w].x - ref);
       L += f * stat[w].y;
       O += f * red[w][threadIdx.x];
     }
@@ -198,13 +174,14 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 2 : 1) cross_direct
       po[c] = load_peer(&part[2 + d], peer);
       M = fmaxf(M, pm[c]);
     }
+    const float ref = M == -CUDART_INF_F ? 0.f : M;
 #pragma unroll
     for (int c = 0; c < kMaxCluster; ++c) {
-      const float f = pm[c] == -CUDART_INF_F ? 0.f : fast_exp2(pm[c] - M);
+      const float f = c < p.C ? fast_exp2(pm[c] - ref) : 0.f;
       L += f * pl[c];
       O += f * po[c];
     }
-    p.out[(size_t)bh * D + d] = L > 0.f ? O / L : 0.f;  // no cached keys: an empty softmax, zero
+    p.out[(size_t)bh * D + d] = M == -CUDART_INF_F ? 0.f : O / L;  // no cached keys: an empty softmax, zero
   }
   cluster_arrive();  // a CTA's shared memory stays until its peers have read it
   cluster_wait();

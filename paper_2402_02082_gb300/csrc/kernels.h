@@ -89,6 +89,9 @@ cudaError_t launch_cross_attn(const AttnArgs& a, cudaStream_t st);
 // Multi-head cross-attention without a workspace; cudaErrorNotSupported where
 // the streaming kernel of launch_cross_attn is the one to take.
 cudaError_t launch_cross_direct(const AttnArgs& a, cudaStream_t st);
+// fp32 tree verification and grouped-query cross-attention without a workspace;
+// cudaErrorNotSupported where launch_tree_attn_fma is the one to take.
+cudaError_t launch_tree_direct(const AttnArgs& a, cudaStream_t st);
 cudaError_t launch_tree_attn_fma(const AttnArgs& a, cudaStream_t st);
 // Returns cudaErrorNotSupported when the tensor-core kernel does not apply to `a`.
 cudaError_t launch_tree_attn_tc(const AttnArgs& a, cudaStream_t st);

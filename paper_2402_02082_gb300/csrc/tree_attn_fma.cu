@@ -9,8 +9,9 @@
 // ancestor-or-self mask on CaPE's trees (proposal spine plus expansion
 // leaves); the kernel takes any parent array.
 //
-// This is the general kernel: any dtype (bf16, fp32), D in {64, 128}.  The
-// tensor-core kernel (tree_attn_tc.cu) replaces it for bf16 where it applies.
+// This is the general kernel: any dtype (bf16, fp32), D in {64, 128}, any bound
+// on the CTAs.  The tensor-core kernels (tree_attn_tc.cu, tree_attn_wide.cu)
+// replace it for bf16 where they apply, tree_direct.cu for fp32.
 // Structure as in cross_attn.cu (persistent split-KV grid, bulk-copy ring,
 // last-CTA merge); here each consumer warp owns a fixed subset of the queries
 // and reads every tile, and the ancestor mask lives in shared memory as one

@@ -75,3 +75,28 @@ def test_cross_paths_agree(B, H, D, dtype, kv, cap):
     for b, h in pairs:
         want[b, 0, h] = oracle.cross_attn(q[b:b + 1, :, h:h + 1], K[b:b + 1, h:h + 1], V[b:b + 1, h:h + 1], [kv[b]])[0, 0, 0]
     assert_attn_close(auto, want, pairs, f"cross B{B} H{H} D{D} {dtype} {kv}")
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_non_finite_scores(dtype):
+    """The direct kernel: a NaN in a key is in its head's output and no other's; keys of score -inf have weight zero,
+    a warp's whole tiles of them too."""
+    B, H, D, n = 2, 4, 64, 300
+    K = synth.normal_values(31, 1, (B, H, n, D), dtype)
+    V = synth.normal_values(31, 2, (B, H, n, D), dtype)
+    q = synth.normal_values(31, 3, (B, 1, H, D), dtype)
+    qd, Kd, Vd, kvd = dev(q), dev(K), dev(V), dev(np.asarray([n, n], np.int32))
+    qd[:, :, 1, 0] = 1.0
+    keep = np.r_[0:16, 80:n]
+    want = oracle.cross_attn(qd.float().cpu().numpy()[:1, :, 1:2], Kd.float().cpu().numpy()[:1, 1:2, keep],
+                             Vd.float().cpu().numpy()[:1, 1:2, keep], [len(keep)])[0, 0, 0]
+    Kd[0, 1, 16:80, 0] = float("-inf")
+    Kd[1, 2, 37, 3] = float("nan")
+    desc = gb.make_desc(B, H, D, n, gb.GLIDE_BF16 if dtype == "bf16" else gb.GLIDE_F32)
+    ws = torch.zeros(gb.glide_attn_workspace_bytes(desc, 1), dtype=torch.uint8, device="cuda")
+    out = torch.zeros((B, 1, H, D), device="cuda")
+    gb.glide_cross_attn(qd, Kd, Vd, kvd, n, out, ws)
+    got = out.cpu().numpy()
+    nan = np.isnan(got).all(-1)[:, 0]
+    assert nan.sum() == 1 and nan[1, 2] and np.isfinite(got[~nan[:, None]]).all()
+    assert np.abs(got[0, 0, 1] - want).max() <= AGREE
