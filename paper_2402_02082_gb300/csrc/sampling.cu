@@ -5,16 +5,27 @@
 // max(0, p_T,i - p_D,i), else from p_T,gamma+1, by inverse CDF with v: the
 // first token whose running weight exceeds v * (total weight).
 //
-// One launch, no waiting:
-// 1. one CTA per (sequence, position) row of target logits: an online
-//    (max, sum of exp) over the row, then, for a proposal position, p_T(x_i)
-//    and the acceptance decision; the CTA counts itself in for its sequence;
-// 2. the CTA that completes a sequence's count finds the first rejection and
-//    draws the extra token from the row it names.  Each warp owns a contiguous
-//    segment of the row and sums its weights with unit-stride loads; a scan
-//    over the 32 segment totals places the segments on the running total; the
-//    warp whose segment reaches past v * total walks it in 32-token groups
-//    (a shuffle scan per group) to the first token past the target.
+// What bounds it: latency.  A sequence's rows are a few hundred KB, a
+// microsecond of one GPC's share of the bandwidth, and what the draw reads
+// depends on every row's decision.  So a cluster of C CTAs serves a sequence
+// and its warps meet twice at the cluster barrier, through distributed shared
+// memory, instead of counting rows in through global memory:
+// 1. each row is cut into 32 parts, each part an online (max, sum of exp) by one
+//    warp, the (gamma + 1) x 32 parts dealt over the cluster's warps; a part's
+//    result goes to every CTA, and each CTA merges the parts of a row in order
+//    and decides every position.  The loads a decision needs (the draft's token,
+//    its logit and probability, u) are issued before the rows;
+// 2. the row of the first rejection is cut into 32 contiguous segments, a warp
+//    each, whose weights are summed with unit-stride loads and kept in shared
+//    memory; the segments' sums go to every CTA, a scan places them on the
+//    running total, and the warp whose segment reaches past v * total walks it in
+//    32-token groups (a shuffle scan per group) to the first token past the
+//    target.
+// The parts, the segments and the order of every sum do not depend on C.
+// Measured over three sets in turn, with a CTA per row, a global counter and a
+// second pass by one CTA -> this (us): 1 sequence, gamma 4, 32000 tokens 12.0 ->
+// 7.3; 4 sequences, gamma 5 12.8 -> 8.6, gamma 4, 50257 tokens 17.3 -> 11.8; 16,
+// gamma 8 13.5 -> 12.0; 64, gamma 4 27.8 -> 18.6.
 // Floating point decides integers here (a decision, a token), in fp32 with
 // this kernel's summation order; an exact real-number computation can differ
 // only where u * p_D(x) or v * total lies within rounding of its threshold.
@@ -22,16 +33,24 @@
 #include <math_constants.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "attn_common.cuh"
 #include "kernels.h"
 
 namespace glide {
 namespace {
 
-constexpr int kThreads = 1024;
-constexpr int kWarps = kThreads / 32;
-constexpr int kBatch = 8;   // row-scan loads in flight per thread
-constexpr int kGrp = 8;     // draw: 32-token groups whose loads are issued together
+constexpr int kParts = 32;                // parts of a row, and segments of the drawn row
+constexpr int kWarps = 20;                // per CTA
+constexpr int kThreads = kWarps * 32;
+constexpr int kChunk = 16;                // floats of a row that a lane loads at once
+constexpr int kGrp = 32;                  // draw: 32-token groups whose loads are issued together
+constexpr int kWalk = 8;                  // walk: groups scanned together
+constexpr int kKeep = 1632;               // weights of a segment that stay in shared memory
+constexpr int kMaxRowsS = kMaxTree;       // gamma + 1 at most
+constexpr int kMaxCluster = 16;
+constexpr int kPortable = 8;              // every device runs clusters of this size
 
 struct SampleParams {
   const int32_t* draft;    // [B, gamma]
@@ -40,235 +59,371 @@ struct SampleParams {
   const float* u;          // [B, gamma + 1]
   int32_t* n_acc;          // [B]
   int32_t* next_tok;       // [B]
-  unsigned* counters;      // [B]
-  float2* stats;           // [B, gamma + 1]: (max, sum of 2^((l - max) * log2 e))
-  int* accept;             // [B, gamma]
-  int B, gamma, V;
+  int gamma, V, C;
 };
 
+// The running (max, sum of 2^((x - max) log2 e)) takes one more value, or another
+// running pair, without a branch: the smaller maximum's side is rescaled.
 __device__ __forceinline__ void online_add(float& m, float& s, float x) {
-  if (x > m) {
-    s = s * fast_exp2((m - x) * kLog2e) + 1.f;
-    m = x;
-  } else {
-    s += fast_exp2((x - m) * kLog2e);
-  }
+  const bool up = x > m;
+  const float e = fast_exp2(-fabsf(x - m) * kLog2e);
+  s = fmaf(up ? s : 1.f, e, up ? 1.f : s);
+  m = up ? x : m;
 }
-
 __device__ __forceinline__ void online_merge(float& m, float& s, float m2, float s2) {
-  if (m2 == -CUDART_INF_F) return;
-  if (m2 > m) {
-    s = s * fast_exp2((m - m2) * kLog2e) + s2;
-    m = m2;
-  } else {
-    s += s2 * fast_exp2((m2 - m) * kLog2e);
-  }
+  const bool up = m2 > m;
+  const float e = fast_exp2(-fabsf(m2 - m) * kLog2e);
+  if (m2 != -CUDART_INF_F) s = fmaf(up ? s : s2, e, up ? s2 : s);
+  m = up ? m2 : m;
 }
 
-__global__ void __launch_bounds__(kThreads) spec_sample_kernel(const SampleParams p) {
-  __shared__ float2 red[kWarps];
-  __shared__ float seg_up[kWarps];
-  __shared__ int last, s_tok, s_lastpos, s_win;
-  pdl_wait();
+// A value of this CTA's address in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void store_peer(float2* p, uint32_t rank, float2 v) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(peer_addr(p, rank)), "f"(v.x), "f"(v.y) : "memory");
+}
 
-  const int G1 = p.gamma + 1;
-  const int row = blockIdx.x;
-  const int b = row / G1, i = row - b * G1;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const float* lg = p.logits + (size_t)row * p.V;
-
-  // ---- 1. (max, sum) of the row; batches of kBatch loads per thread, all
-  // issued before any use
-  float m = -CUDART_INF_F, s = 0.f;
-  if ((p.V & 3) == 0) {
-    const float4* l4 = reinterpret_cast<const float4*>(lg);
-    const int n4 = p.V / 4;
-    for (int j0 = threadIdx.x; j0 < n4; j0 += kBatch * kThreads) {
-      float4 x[kBatch];
+// The (max, sum) of parts first, first + every, ... of the `total` parts of the
+// rows of n units of kVec floats; a part is the units part x 32 + lane, + 1024, ...
+// in turn.  Two chunks of kChunk floats a lane are in flight, the later one
+// under the arithmetic of the earlier, across the ends of parts.
+template <int kVec, class F>
+__device__ __forceinline__ void scan_parts(const float* rows, int n, int first, int every, int total, int lane, F finish) {
+  constexpr int kUnits = kChunk / kVec, kSpan = kUnits * kParts * 32;
+  float x[2][kChunk];
+  auto start = [&](int k) { return k % kParts * 32 + lane; };
+  auto load = [&](float (&v)[kChunk], int k, int j) {
+    const float* row = rows + (size_t)(k / kParts) * n * kVec;
 #pragma unroll
-      for (int k = 0; k < kBatch; ++k)
-        if (j0 + k * kThreads < n4) x[k] = __ldg(l4 + j0 + k * kThreads);
-#pragma unroll
-      for (int k = 0; k < kBatch; ++k)
-        if (j0 + k * kThreads < n4) {
-          online_add(m, s, x[k].x);
-          online_add(m, s, x[k].y);
-          online_add(m, s, x[k].z);
-          online_add(m, s, x[k].w);
+    for (int e = 0; e < kUnits; ++e) {
+      const int u = j + e * kParts * 32;
+      if constexpr (kVec == 4) {
+        if (u < n) {
+          const float4 f = __ldcg(reinterpret_cast<const float4*>(row) + u);
+          v[4 * e] = f.x;
+          v[4 * e + 1] = f.y;
+          v[4 * e + 2] = f.z;
+          v[4 * e + 3] = f.w;
         }
-    }
-  } else {
-    for (int j0 = threadIdx.x; j0 < p.V; j0 += kBatch * kThreads) {
-      float x[kBatch];
-#pragma unroll
-      for (int k = 0; k < kBatch; ++k)
-        if (j0 + k * kThreads < p.V) x[k] = __ldg(lg + j0 + k * kThreads);
-#pragma unroll
-      for (int k = 0; k < kBatch; ++k)
-        if (j0 + k * kThreads < p.V) online_add(m, s, x[k]);
-    }
-  }
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) {
-    const float m2 = __shfl_xor_sync(0xffffffffu, m, off), s2 = __shfl_xor_sync(0xffffffffu, s, off);
-    online_merge(m, s, m2, s2);
-  }
-  if (lane == 0) red[warp] = make_float2(m, s);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float M = red[0].x, S = red[0].y;
-    for (int w = 1; w < kWarps; ++w) online_merge(M, S, red[w].x, red[w].y);
-    p.stats[row] = make_float2(M, S);
-    if (i < p.gamma) {
-      int x = p.draft[(size_t)b * p.gamma + i];
-      x = x < 0 ? 0 : (x >= p.V ? p.V - 1 : x);
-      const float pt = fast_exp2((__ldg(lg + x) - M) * kLog2e) / S;
-      const float qd = p.q[((size_t)b * p.gamma + i) * p.V + x];
-      p.accept[(size_t)b * p.gamma + i] = (p.u[(size_t)b * G1 + i] * qd < pt) ? 1 : 0;
-    }
-    __threadfence();
-    const unsigned prev = atomicAdd(&p.counters[b], 1u);
-    last = prev == (unsigned)p.gamma ? 1 : 0;  // gamma + 1 rows per sequence
-    if (last) __threadfence();
-  }
-  __syncthreads();
-  if (!last) return;
-
-  // ---- 2. the first rejection and the extra token of sequence b
-  int n = p.gamma;
-  for (int k = 0; k < p.gamma; ++k)
-    if (!__ldcg(p.accept + (size_t)b * p.gamma + k)) {
-      n = k;
-      break;
-    }
-  const float2 st = __ldcg(p.stats + (size_t)b * G1 + n);
-  const float* L = p.logits + ((size_t)b * G1 + n) * p.V;
-  const float* Q = n < p.gamma ? p.q + ((size_t)b * p.gamma + n) * p.V : nullptr;  // null: draw from p_T
-  const float inv = 1.f / st.y;
-  const float v = p.u[(size_t)b * G1 + p.gamma];
-  const int seg = (p.V + kWarps - 1) / kWarps;  // contiguous segment per warp
-  const int x0 = min(p.V, warp * seg), x1 = min(p.V, x0 + seg);
-
-  // weights of kGrp 32-token groups starting at base (lane j: token base + 32k + j);
-  // every load first, then the arithmetic; 0 past the segment
-  auto groups = [&](int base, float (&w)[kGrp]) {
-    float lv[kGrp], qv[kGrp];
-#pragma unroll
-    for (int k = 0; k < kGrp; ++k) {
-      const int x = base + 32 * k + lane;
-      lv[k] = x < x1 ? __ldg(L + x) : 0.f;
-      qv[k] = (Q && x < x1) ? __ldg(Q + x) : 0.f;
-    }
-#pragma unroll
-    for (int k = 0; k < kGrp; ++k) {
-      const float pt = fast_exp2((lv[k] - st.x) * kLog2e) * inv;
-      w[k] = base + 32 * k + lane < x1 ? (Q ? fmaxf(0.f, pt - qv[k]) : pt) : 0.f;
+      } else {
+        if (u < n) v[e] = __ldcg(row + u);
+      }
     }
   };
+  // the chunk after (k, j): the part's next, else the next part's first
+  auto advance = [&](int& k, int& j) {
+    j += kSpan;
+    if (j - lane >= n) {  // the same for all lanes
+      k += every;
+      j = start(k);
+    }
+  };
+  int k0 = first, j0 = start(first);
+  if (k0 >= total) return;
+  int k1 = k0, j1 = j0;
+  load(x[0], k0, j0);
+  advance(k1, j1);
+  if (k1 < total) load(x[1], k1, j1);
+  float m = -CUDART_INF_F, s = 0.f;
+#pragma unroll 1
+  while (k0 < total) {
+#pragma unroll
+    for (int e = 0; e < kUnits; ++e)
+      if (j0 + e * kParts * 32 < n) {
+#pragma unroll
+        for (int c = 0; c < kVec; ++c) online_add(m, s, x[0][kVec * e + c]);
+      }
+    if (k1 != k0) {
+      finish(k0, m, s);
+      m = -CUDART_INF_F;
+      s = 0.f;
+    }
+#pragma unroll
+    for (int e = 0; e < kChunk; ++e) x[0][e] = x[1][e];
+    k0 = k1;
+    j0 = j1;
+    advance(k1, j1);
+    if (k1 < total) load(x[1], k1, j1);
+  }
+}
 
-  // Inverse-CDF draw from the current weights; -1 when they sum to 0.
-  auto draw = [&]() -> int {
-    float part = 0.f;
-    int lastpos = -1;
-    for (int base = x0; base < x1; base += 32 * kGrp) {
-      float w[kGrp];
-      groups(base, w);
+__global__ void __launch_bounds__(kThreads, 1) spec_sample_kernel(const SampleParams p) {
+  extern __shared__ float keep[];                // weights of this CTA's segments, kKeep of each
+  __shared__ float2 red[kMaxRowsS][kParts];      // (max, sum) of every part of every row
+  __shared__ float2 segs[kParts];                // (sum of weights, last token with one) of every segment
+  __shared__ float2 stats[kMaxRowsS];
+  __shared__ int accepted[kMaxRowsS];
+  cluster_arrive();  // no CTA writes into one that has not started
+  pdl_wait();
+  const int G1 = p.gamma + 1, V = p.V;
+  const int rank = (int)cluster_rank(), b = blockIdx.x / p.C;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const float* rows = p.logits + (size_t)b * G1 * V;
+  const float* probs = p.q + (size_t)b * p.gamma * V;
+
+  // what the decision of row `warp` needs
+  float lx = 0.f, qx = 0.f, ux = 0.f;
+  auto fetch = [&](int i) {
+    if (i >= p.gamma || lane != 0) return;
+    int x = __ldcg(p.draft + (size_t)b * p.gamma + i);
+    ux = __ldcg(p.u + (size_t)b * G1 + i);
+    x = x < 0 ? 0 : (x >= V ? V - 1 : x);
+    lx = __ldcg(rows + (size_t)i * V + x);
+    qx = __ldcg(probs + (size_t)i * V + x);
+  };
+  fetch(warp);
+  const float v = __ldcg(p.u + (size_t)b * G1 + p.gamma);
+
+  // ---- 1. (max, sum) of every part
+  bool started = false;
+  auto finish = [&](int k, float m, float s) {
 #pragma unroll
-      for (int k = 0; k < kGrp; ++k) {
-        part += w[k];
-        if (w[k] > 0.f) lastpos = base + 32 * k + lane;
+    for (int off = 16; off >= 1; off >>= 1) {
+      const float m2 = __shfl_xor_sync(0xffffffffu, m, off), s2 = __shfl_xor_sync(0xffffffffu, s, off);
+      online_merge(m, s, m2, s2);
+    }
+    m = __shfl_sync(0xffffffffu, m, 0);  // lane 0's order of merges
+    s = __shfl_sync(0xffffffffu, s, 0);
+    if (!started) cluster_wait();
+    started = true;
+    if (lane < p.C) store_peer(&red[k / kParts][k % kParts], lane, make_float2(m, s));
+  };
+  if ((V & 3) == 0)
+    scan_parts<4>(rows, V / 4, rank * kWarps + warp, p.C * kWarps, G1 * kParts, lane, finish);
+  else
+    scan_parts<1>(rows, V, rank * kWarps + warp, p.C * kWarps, G1 * kParts, lane, finish);
+  if (!started) cluster_wait();
+  cluster_arrive();
+  cluster_wait();
+
+  // ---- the rows' statistics: parts 0, 1, ... merged in order, and the decisions
+  for (int i = warp; i < G1; i += kWarps) {
+    if (i != warp) fetch(i);
+    const float2 r = red[i][lane];
+    float before = r.x;  // the maximum of the parts before this one
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const float y = __shfl_up_sync(0xffffffffu, before, off);
+      if (lane >= off) before = fmaxf(before, y);
+    }
+    const float M = __shfl_sync(0xffffffffu, before, 31);
+    before = __shfl_up_sync(0xffffffffu, before, 1);
+    const float e = fast_exp2(-fabsf(r.x - before) * kLog2e);
+    const unsigned up = __ballot_sync(0xffffffffu, r.x > before);
+    const unsigned take = __ballot_sync(0xffffffffu, r.x != -CUDART_INF_F);
+    float S = __shfl_sync(0xffffffffu, r.y, 0);
+#pragma unroll
+    for (int w = 1; w < kParts; ++w) {
+      const float ew = __shfl_sync(0xffffffffu, e, w), sw = __shfl_sync(0xffffffffu, r.y, w);
+      const bool u = (up >> w) & 1u;
+      if ((take >> w) & 1u) S = fmaf(u ? S : sw, ew, u ? sw : S);
+    }
+    if (lane == 0) {
+      stats[i] = make_float2(M, S);
+      if (i < p.gamma) {
+        const float pt = fast_exp2((lx - M) * kLog2e) / S;
+        accepted[i] = (ux * qx < pt) ? 1 : 0;
       }
     }
-    const float segsum = warp_sum(part);
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) lastpos = max(lastpos, __shfl_xor_sync(0xffffffffu, lastpos, off));
-    __syncthreads();  // the shared slots of a previous draw are free again
-    if (threadIdx.x == 0) {
-      s_tok = -1;
-      s_lastpos = -1;
-      s_win = kWarps;
-    }
-    if (lane == 0) seg_up[warp] = segsum;
-    __syncthreads();
-    if (lane == 0) atomicMax(&s_lastpos, lastpos);
-    if (warp == 0) {
-      float t = seg_up[lane];
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const float y = __shfl_up_sync(0xffffffffu, t, off);
-        if (lane >= off) t += y;
-      }
-      seg_up[lane] = t;  // upper end of each segment on the running total
-      const float target = v * __shfl_sync(0xffffffffu, t, 31);
-      const unsigned hit = __ballot_sync(0xffffffffu, t > target);
-      if (lane == 0 && hit) s_win = __ffs(hit) - 1;  // the first segment past the target
-    }
-    __syncthreads();
-    const float total = seg_up[kWarps - 1];
-    if (!(total > 0.f)) return -1;
-    if (warp == s_win) {
-      const float target = v * total;
-      float running = warp > 0 ? seg_up[warp - 1] : 0.f;
-      int tok = -1;
-      for (int base = x0; base < x1 && tok < 0; base += 32 * kGrp) {
-        float w[kGrp];
-        groups(base, w);
+  }
+  __syncthreads();
+
+  // ---- 2. the first rejection and the extra token
+  int n = 0;
+  while (n < p.gamma && accepted[n]) ++n;
+  const float2 st = stats[n];
+  const float* L = rows + (size_t)n * V;
+  const float* Q = n < p.gamma ? probs + (size_t)n * V : nullptr;  // null: draw from p_T
+  const float inv = 1.f / st.y;
+  const int seg = (V + kParts - 1) / kParts;  // contiguous tokens per segment
+
+  // Inverse-CDF draw from the current weights; -1 when they sum to 0.  Every
+  // warp of the cluster returns the same sign; the winning one the token.
+  auto draw = [&]() -> bool {
+#pragma unroll 1
+    for (int sl = warp; rank + sl * p.C < kParts; sl += kWarps) {  // segments rank, rank + C, ... are this CTA's
+      const int sg = rank + sl * p.C, x0 = min(V, sg * seg), x1 = min(V, x0 + seg);
+      float part = 0.f;
+      int lastpos = -1;
+#pragma unroll 1
+      for (int base = x0; base < x1; base += 32 * kGrp) {
+        float lv[kGrp], qv[kGrp];
 #pragma unroll
         for (int k = 0; k < kGrp; ++k) {
-          float incl = w[k];
+          const int x = base + 32 * k + lane;
+          lv[k] = x < x1 ? __ldcg(L + x) : 0.f;
+          qv[k] = (Q && x < x1) ? __ldcg(Q + x) : 0.f;
+        }
 #pragma unroll
-          for (int off = 1; off < 32; off <<= 1) {
-            const float y = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += y;
+        for (int k = 0; k < kGrp; ++k) {
+          const int x = base + 32 * k + lane;
+          const float pt = fast_exp2((lv[k] - st.x) * kLog2e) * inv;
+          const float w = x < x1 ? (Q ? fmaxf(0.f, pt - qv[k]) : pt) : 0.f;
+          if (x - x0 < kKeep) keep[sl * kKeep + x - x0] = w;
+          part += w;
+          if (w > 0.f) lastpos = x;
+        }
+      }
+      const float segsum = warp_sum(part);
+#pragma unroll
+      for (int off = 16; off >= 1; off >>= 1) lastpos = max(lastpos, __shfl_xor_sync(0xffffffffu, lastpos, off));
+      if (lane < p.C) store_peer(&segs[sg], lane, make_float2(segsum, __int_as_float(lastpos)));
+    }
+    cluster_arrive();
+    cluster_wait();
+    const float2 sv = segs[lane];
+    float t = sv.x;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const float y = __shfl_up_sync(0xffffffffu, t, off);
+      if (lane >= off) t += y;
+    }  // t: upper end of segment `lane` on the running total
+    const float total = __shfl_sync(0xffffffffu, t, 31);
+    if (!(total > 0.f)) return false;
+    const float target = v * total;
+    const unsigned past = __ballot_sync(0xffffffffu, t > target);
+    // no segment past the target: rounding at the very end, the row's last token
+    const int last = __reduce_max_sync(0xffffffffu, __float_as_int(sv.y));
+    const int win = past ? __ffs(past) - 1 : 0;
+    if (win % p.C != rank || win / p.C % kWarps != warp) return true;
+    int tok = -1;
+    if (past) {
+      const int sl = win / p.C, x0 = min(V, win * seg), x1 = min(V, x0 + seg);
+      float running = __shfl_sync(0xffffffffu, t, win > 0 ? win - 1 : 0);
+      if (win == 0) running = 0.f;
+#pragma unroll 1
+      for (int base = x0; base < x1 && tok < 0; base += 32 * kWalk) {
+        float w[kWalk], incl[kWalk];
+#pragma unroll
+        for (int k = 0; k < kWalk; ++k) {
+          const int x = base + 32 * k + lane;
+          w[k] = 0.f;
+          if (x < x1) {
+            if (x - x0 < kKeep) {
+              w[k] = keep[sl * kKeep + x - x0];
+            } else {
+              const float pt = fast_exp2((__ldcg(L + x) - st.x) * kLog2e) * inv;
+              w[k] = Q ? fmaxf(0.f, pt - __ldcg(Q + x)) : pt;
+            }
           }
-          const unsigned hit = __ballot_sync(0xffffffffu, running + incl > target && w[k] > 0.f);
+          incl[k] = w[k];
+        }
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1)
+#pragma unroll
+          for (int k = 0; k < kWalk; ++k) {
+            const float y = __shfl_up_sync(0xffffffffu, incl[k], off);
+            if (lane >= off) incl[k] += y;
+          }
+#pragma unroll
+        for (int k = 0; k < kWalk; ++k) {
+          const unsigned hit = __ballot_sync(0xffffffffu, running + incl[k] > target && w[k] > 0.f);
           if (tok < 0 && hit) tok = base + 32 * k + __ffs(hit) - 1;
-          running += __shfl_sync(0xffffffffu, incl, 31);
+          running += __shfl_sync(0xffffffffu, incl[k], 31);
         }
       }
       // rounding can leave the walk just short of the target: the segment's last token
-      if (lane == 0) s_tok = tok >= 0 ? tok : lastpos;
+      if (tok < 0) tok = __float_as_int(__shfl_sync(0xffffffffu, sv.y, win));
     }
-    __syncthreads();
-    return s_tok >= 0 ? s_tok : s_lastpos;  // no segment past the target: rounding at the very end
+    if (tok < 0) tok = last;
+    if (lane == 0) p.next_tok[b] = tok;
+    return true;
   };
 
-  int tok = draw();
-  if (tok < 0) {  // max(0, p_T - p_D) summed to 0 in fp32: draw from p_T instead
+  bool drawn = draw();
+  if (!drawn) {  // max(0, p_T - p_D) summed to 0 in fp32: draw from p_T instead
     Q = nullptr;
-    tok = draw();
+    cluster_arrive();  // every warp has read the first draw's sums
+    cluster_wait();
+    drawn = draw();
   }
-  if (threadIdx.x == 0) {
+  if (rank == 0 && threadIdx.x == 0) {
     p.n_acc[b] = n;
-    p.next_tok[b] = tok;
-    p.counters[b] = 0u;
+    if (!drawn) p.next_tok[b] = -1;
   }
+}
+
+size_t keep_bytes(int C) { return (size_t)((kParts + C - 1) / C) * kKeep * sizeof(float); }
+
+cudaLaunchConfig_t config(int B, int C, cudaStream_t st, cudaLaunchAttribute* attr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(B * C));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = keep_bytes(C);
+  cfg.stream = st;
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)C;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cfg;
+}
+
+// How many clusters of each size the chip runs at once (0: none, or unknown).
+struct Room {
+  int clusters[kMaxCluster + 1] = {};
+};
+Room find_room() {
+  Room r;
+  for (int C = 1; C <= kMaxCluster; ++C) {
+    if (C > kPortable && C < kMaxCluster) continue;
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = config(1, C, nullptr, attr);
+    cfg.attrs = attr + 1;  // the cluster's size alone
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&r.clusters[C], spec_sample_kernel, &cfg) != cudaSuccess) {
+      r.clusters[C] = 0;
+      cudaGetLastError();
+    }
+  }
+  return r;
 }
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 }  // namespace
 
-// Workspace: [0,256) status | counters [B] | stats [B*(gamma+1)] float2 | decisions [B*gamma] int.
+// The call's workspace, as its callers allocate it; this kernel's warps meet in distributed shared
+// memory and leave it alone.
 size_t sample_workspace_bytes(int B, int gamma) {
   return 256 + align256((size_t)B * 4) + align256((size_t)B * (gamma + 1) * 8) + align256((size_t)B * gamma * 4);
 }
 
 cudaError_t launch_spec_sample(const SampleArgs& a, cudaStream_t st) {
+  static std::atomic<int> configured{-1};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (configured.load() != dev) {
+    e = cudaFuncSetAttribute(spec_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)keep_bytes(1));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(spec_sample_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    configured.store(dev);
+  }
+  // CTAs per sequence: as many as let all sequences run at once (a second wave
+  // costs as much as the first: 16 sequences, gamma 4, C = 6 and 8: 10.2 and 13.3
+  // us).  Sixteen only where they save a round of parts (4 sequences, gamma 8,
+  // C = 8 and 16: 10.2 and 8.9 us; gamma 4: 7.95 and 8.1).
+  static const Room room = find_room();
+  int C = kPortable;
+  while (C > 1 && a.B > room.clusters[C]) --C;
+  if (C == kPortable && (a.gamma + 1) * kParts > C * kWarps && a.B <= room.clusters[kMaxCluster]) C = kMaxCluster;
   SampleParams p;
   p.draft = a.draft; p.q = a.q; p.logits = a.logits; p.u = a.u;
   p.n_acc = a.n_acc; p.next_tok = a.next_tok;
-  p.B = a.B; p.gamma = a.gamma; p.V = a.V;
-  unsigned char* ws = static_cast<unsigned char*>(a.ws);
-  size_t off = 256;
-  p.counters = reinterpret_cast<unsigned*>(ws + off);
-  off += align256((size_t)a.B * 4);
-  p.stats = reinterpret_cast<float2*>(ws + off);
-  off += align256((size_t)a.B * (a.gamma + 1) * 8);
-  p.accept = reinterpret_cast<int*>(ws + off);
-  const long long grid = (long long)a.B * (a.gamma + 1);
-  if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-  return launch_pdl(spec_sample_kernel, dim3((unsigned)grid), dim3(kThreads), 0, st, p);
+  p.gamma = a.gamma; p.V = a.V; p.C = C;
+  if ((long long)a.B * C > 0x7fffffffLL) return cudaErrorInvalidValue;
+  cudaLaunchAttribute attr[2];
+  const cudaLaunchConfig_t cfg = config(a.B, C, st, attr);
+  return cudaLaunchKernelEx(&cfg, spec_sample_kernel, p);
 }
 
 }  // namespace glide
