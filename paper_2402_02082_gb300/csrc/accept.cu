@@ -27,6 +27,13 @@
 // order, sequence b's chunks are all read before sequence b + 1's, and warps
 // count their chunks while they wait for the next one: the walks of the early
 // sequences run while the later ones still stream.
+//
+// What bounds it: HBM and, for a few rows, the chain of a launch, a load, the
+// count and the walk (~4 us).  Rows of any length come by bulk copy (Span), and
+// the code is a loop with one wait, one scan and one walk in it (22 KB; 50 with
+// a copy of the walk at every place that counts).  4 x 64 rows, us, with rows of
+// odd length read by plain loads -> this: 32000 tokens 8.4 -> 8.1, 32001 19.7 ->
+// 8.1, 50257 36.4 -> 12.2; one row of 32001 8.9 -> 3.8.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -46,6 +53,13 @@ constexpr size_t kSmemBytes = kRingBytes + 2 * kNS * sizeof(uint64_t) + 16;
 static_assert(kNS % kNW == 0, "a stage must always serve the same consumer warp");
 static_assert(kMaxTree <= 64, "two tree nodes per lane");
 
+// A chunk: split `split` of node `node` of sequence `seq`.  Chunks are numbered in
+// that order; a Step is a distance in it (split < splits, node < n), so that the
+// roles walk their chunks without a division.
+struct Step {
+  int seq, node, split;
+};
+
 struct AccParams {
   const int32_t* draft;
   const int32_t* parent;
@@ -57,8 +71,7 @@ struct AccParams {
   unsigned* counters;
   unsigned long long* slots;
   int B, n, V, splits;
-  long long nchunks;  // B * n * splits
-  int bulk;           // 1: rows start 16-byte aligned, chunks arrive by bulk copy; 0: consumers read global memory
+  Step one, round;    // to the CTA's next chunk (G chunks on), to a consumer warp's (kNW G)
 };
 
 __device__ __forceinline__ unsigned long long argmax_key(float f, int idx) {
@@ -92,15 +105,21 @@ __device__ __forceinline__ unsigned long long warp_max_key(unsigned long long k)
 // a warp barrier) are visible before any write after it.
 __device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
+__device__ __forceinline__ void mask_head(float4& v, int head) {
+  if (head > 0) v.x = -__int_as_float(0x7f800000);
+  if (head > 1) v.y = -__int_as_float(0x7f800000);
+  if (head > 2) v.z = -__int_as_float(0x7f800000);
+}
+
 // One lane's part of a chunk in shared memory: the float4 groups lane,
-// lane + 32, ... below n4 (all kGroups of them when kFull).  Groups are loaded
+// lane + 32, ... below n4.  Groups are loaded
 // eight at a time into eight independent chains (group i goes to chain
 // i % 8); a strict comparison keeps the first group of each chain holding the
 // chain's maximum, and the chains are combined lowest group first among equal
-// maxima.  Returns the lane's maximum and the group holding its first
-// occurrence (-1 when the lane has no group).
-template <bool kFull>
-__device__ __forceinline__ int scan_lane(const float4* s4, int n4, int lane, float& best) {
+// maxima.  The first `head` floats of group 0 are not the chunk's.  Returns the
+// lane's maximum and the group holding its first occurrence (-1 when the lane has
+// no group).
+__device__ __forceinline__ int scan_lane(const float4* s4, int n4, int lane, int head, float& best) {
   constexpr int kC = 8;
   float acc[kC];
   int grp[kC];
@@ -115,14 +134,15 @@ __device__ __forceinline__ int scan_lane(const float4* s4, int n4, int lane, flo
 #pragma unroll
     for (int j = 0; j < kC; ++j) {
       const int q = lane + 32 * (b * kC + j);
-      if (kFull || q < n4) v[j] = s4[q];
+      if (q < n4) v[j] = s4[q];
     }
+    if (b == 0 && lane == 0) mask_head(v[0], head);
 #pragma unroll
     for (int j = 0; j < kC; ++j) {
       const int q = lane + 32 * (b * kC + j);
-      if (kFull || q < n4) {
+      if (q < n4) {
         const float g = fmaxf(fmaxf(v[j].x, v[j].y), fmaxf(v[j].z, v[j].w));
-        if (b == 0 || grp[j] < 0 || g > acc[j]) {
+        if (grp[j] < 0 || g > acc[j]) {
           acc[j] = g;
           grp[j] = b * kC + j;
         }
@@ -232,6 +252,48 @@ __device__ void walk_tree(const AccParams& p, int b, int lane) {
   if (h1) p.slots[base + c1] = 0ull;
 }
 
+// What a bulk copy takes of a chunk: it wants 16-byte boundaries, and rows start
+// on them only where V is a multiple of 4.  So the copy begins up to three floats
+// before the chunk (`head`: the row before, never before the first row) and ends
+// up to three before its end (`tail`: lanes load those, so that nothing past the
+// logits is read).
+struct Span {
+  size_t first;  // element the copy starts at
+  int head, n4, tail;
+};
+__device__ __forceinline__ Span span_of(const AccParams& p, const Step& c, int cnt) {
+  Span s;
+  const size_t at = ((size_t)c.seq * p.n + c.node) * p.V + (size_t)c.split * kChunk;
+  s.head = (int)(at & 3);
+  s.first = at - s.head;
+  s.n4 = (s.head + cnt) >> 2;
+  s.tail = (s.head + cnt) & 3;
+  return s;
+}
+
+// Distance of chunk k from chunk 0; the chunk after a distance.
+__host__ __device__ __forceinline__ Step step_of(unsigned k, int n, int splits) {
+  const unsigned row = k / (unsigned)splits;
+  Step d;
+  d.split = (int)(k - row * (unsigned)splits);
+  d.seq = (int)(row / (unsigned)n);
+  d.node = (int)(row - (unsigned)d.seq * (unsigned)n);
+  return d;
+}
+__device__ __forceinline__ void advance(Step& c, const Step& d, int n, int splits) {
+  c.split += d.split;
+  c.node += d.node;
+  c.seq += d.seq;
+  if (c.split >= splits) {
+    c.split -= splits;
+    ++c.node;
+  }
+  if (c.node >= n) {
+    c.node -= n;
+    ++c.seq;
+  }
+}
+
 __global__ void __launch_bounds__(kThreads, 1) tree_accept_kernel(const AccParams p) {
   extern __shared__ __align__(1024) unsigned char smem[];
   float* ring = reinterpret_cast<float*>(smem);
@@ -265,24 +327,32 @@ __global__ void __launch_bounds__(kThreads, 1) tree_accept_kernel(const AccParam
       }
       return;
     }
-    if (!p.bulk) return;
     const uint64_t pol = policy_evict_first();
-    long long issued = 0;
-    bool ok = true;
-    for (long long k = c; k < p.nchunks; k += G, ++issued) {
-      const int s = (int)(issued % kNS);
-      const uint32_t use = (uint32_t)(issued / kNS);
-      if (!mbar_wait(&empty[s], (use & 1u) ^ 1u, abort_flag, p.status)) { ok = false; break; }
-      const long long row = k / p.splits;
-      const int lo = (int)(k - row * p.splits) * kChunk;
-      const int cnt = min(kChunk, p.V - lo);
-      const uint32_t bytes = (uint32_t)cnt * 4u;
-      mbar_arrive_expect_tx(&full[s], bytes);
-      bulk_g2s(ring + (size_t)s * kChunk, p.logits + (size_t)row * p.V + lo, bytes, &full[s], pol);
+    Step k = step_of(blockIdx.x, p.n, p.splits);
+    int s = 0, issued = 0;
+    uint32_t phase = 1;
+#pragma unroll 1
+    for (; (unsigned)k.seq < (unsigned)p.B; advance(k, p.one, p.n, p.splits)) {
+      if (!mbar_wait_small(&empty[s], phase, abort_flag)) {
+        record_status(p.status, kStatusTimeout);
+        // let copies already issued land before the CTA exits: the last one of every stage
+        for (int j = 0; j < kNS && j < issued; ++j) mbar_drain(&full[j], (j < s ? phase : phase ^ 1u) ^ 1u);
+        return;
+      }
+      const int cnt = min(kChunk, p.V - k.split * kChunk);
+      const Span sp = span_of(p, k, cnt);
+      if (sp.n4 == 0) {  // all of the chunk is tail
+        mbar_arrive(&full[s]);
+      } else {
+        mbar_arrive_expect_tx(&full[s], (uint32_t)sp.n4 * 16u);
+        bulk_g2s(ring + (size_t)s * kChunk, p.logits + sp.first, (uint32_t)sp.n4 * 16u, &full[s], pol);
+      }
+      issued = issued < kNS ? issued + 1 : kNS;
+      if (++s == kNS) {
+        s = 0;
+        phase ^= 1u;
+      }
     }
-    if (!ok)  // let copies already issued land before the CTA exits
-      for (long long j = (issued > kNS ? issued - kNS : 0); j < issued; ++j)
-        mbar_drain(&full[j % kNS], (uint32_t)(j / kNS) & 1u);
     return;
   }
 
@@ -309,49 +379,45 @@ __global__ void __launch_bounds__(kThreads, 1) tree_accept_kernel(const AccParam
     }
     npend = 0;
   };
-  long long use = 0;  // chunks this warp has taken from its stage
-  for (long long j = warp; c + j * G < p.nchunks; j += kNW, ++use) {
-    const long long k = c + j * G;
-    const long long row = k / p.splits;
-    const int lo = (int)(k - row * p.splits) * kChunk;
+  uint32_t phase = 0;
+  Step k = step_of(blockIdx.x + warp * gridDim.x, p.n, p.splits);
+#pragma unroll 1
+  for (;; advance(k, p.round, p.n, p.splits), phase ^= 1u) {
+    const bool more = (unsigned)k.seq < (unsigned)p.B;
+    if (npend > 0 && (npend == 32 || !more || !__all_sync(0xffffffffu, mbar_test_wait(&full[warp], phase)))) count_in();
+    if (!more) break;
+    const int lo = k.split * kChunk;
     const int cnt = min(kChunk, p.V - lo);
     float m = -__int_as_float(0x7f800000);  // -inf
     int idx = 0x7fffffff;                   // a lane that holds no logit never wins
-    if (p.bulk) {
-      if (npend > 0 && !mbar_test_wait(&full[warp], (uint32_t)(use & 1))) count_in();
-      if (!mbar_wait(&full[warp], (uint32_t)(use & 1), abort_flag, p.status)) break;
-      const float4* s4 = reinterpret_cast<const float4*>(ring + (size_t)warp * kChunk);
-      const int n4 = cnt >> 2;  // cnt is a multiple of 4 in this mode
-      float ma;
-      const int ga = n4 == kChunk / 4 ? scan_lane<true>(s4, n4, lane, ma) : scan_lane<false>(s4, n4, lane, ma);
-      if (ga >= 0) {  // the index inside the winning group
-        const float4 v = s4[lane + 32 * ga];
-        const int e = v.x == ma ? 0 : (v.y == ma ? 1 : (v.z == ma ? 2 : 3));
-        m = ma;
-        idx = lo + 4 * (lane + 32 * ga) + e;
-      }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&empty[warp]);
-    } else {
-      const float* src = p.logits + (size_t)row * p.V + lo;
-      if (lane < cnt) {
-        m = __ldcs(src + lane);
-        idx = lo + lane;
-        for (int q = lane + 32; q < cnt; q += 32) {
-          const float x = __ldcs(src + q);
-          if (x > m) {
-            m = x;
-            idx = lo + q;
-          }
-        }
-      }
+    const Span sp = span_of(p, k, cnt);
+    const bool has_last = lane < sp.tail && 4 * sp.n4 + lane >= sp.head;
+    const float last = has_last ? __ldcg(p.logits + sp.first + 4 * sp.n4 + lane) : 0.f;
+    if (!warp_wait_small(&full[warp], phase, abort_flag)) {
+      if (lane == 0) record_status(p.status, kStatusTimeout);
+      break;
     }
+    const float4* s4 = reinterpret_cast<const float4*>(ring + (size_t)warp * kChunk);
+    float ma;
+    const int ga = scan_lane(s4, sp.n4, lane, sp.head, ma);
+    if (ga >= 0) {  // the index inside the winning group
+      const int q = lane + 32 * ga, h = q == 0 ? sp.head : 0;
+      const float4 v = s4[q];
+      const int e = h < 1 && v.x == ma ? 0 : (h < 2 && v.y == ma ? 1 : (h < 3 && v.z == ma ? 2 : 3));
+      m = ma;
+      idx = lo + 4 * q + e - sp.head;
+    }
+    if (has_last && (idx == 0x7fffffff || last > m)) {
+      m = last;
+      idx = lo - sp.head + 4 * sp.n4 + lane;
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&empty[warp]);
     const unsigned long long key = warp_max_key(argmax_key(m, idx));
-    if (lane == 0) atomicMax(&p.slots[row], key);
-    if (lane == npend) pend_seq = (int)(row / p.n);
-    if (++npend == 32) count_in();
+    if (lane == 0) atomicMax(&p.slots[(size_t)k.seq * p.n + k.node], key);
+    if (lane == npend) pend_seq = k.seq;
+    ++npend;
   }
-  if (npend > 0) count_in();
 }
 
 size_t counters_bytes(int B) { return ((size_t)B * sizeof(unsigned) + 255) & ~size_t(255); }
@@ -381,11 +447,12 @@ cudaError_t launch_tree_accept(const AcceptArgs& a, cudaStream_t st) {
   p.slots = reinterpret_cast<unsigned long long*>(ws + 256 + counters_bytes(a.B));
   p.B = a.B; p.n = a.n; p.V = a.V;
   p.splits = (a.V + kChunk - 1) / kChunk;
-  p.nchunks = (long long)a.B * a.n * p.splits;
-  p.bulk = ((a.V & 3) == 0 && (reinterpret_cast<uintptr_t>(a.logits) & 15u) == 0) ? 1 : 0;
+  const long long nchunks = (long long)a.B * a.n * p.splits;
   if ((long long)a.n * p.splits > 0x7fffffffLL) return cudaErrorInvalidValue;
   long long G = sm_count();
-  if (G > p.nchunks) G = p.nchunks;
+  if (G > nchunks) G = nchunks;
+  p.one = step_of((unsigned)G, a.n, p.splits);
+  p.round = step_of((unsigned)(G * kNW), a.n, p.splits);
   return launch_pdl(tree_accept_kernel, dim3((unsigned)G), dim3(kThreads), kSmemBytes, st, p);
 }
 
