@@ -397,10 +397,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int plen = bt.plen[s.b], len = bt.len[s.b];
       const long long orow = row_at(s);
 
-      // the ancestor-or-self set of this row's tree node, found when the first
-      // tile with tree keys comes (prefix only: no tree keys)
+      // the ancestor-or-self set of this row's tree node, if the segment has tree
+      // keys, while its first keys are on their way
       uint64_t anc = 0;
-      bool anc_ready = !p.tree;
+      if (p.tree && s.t1 * kTK > plen) anc = ancestors(p.parent + (size_t)s.b * n, n, node, valid, lane);
 
       float m_used = -CUDART_INF_F, l = 0.f;  // l: this thread's share of the row sum
       // S of the next tile is loaded while this tile's exponentials run (within
@@ -429,10 +429,6 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int k = 0; k < 16; ++k) sc[k] = __uint_as_float(cur[k]) * sl2;
         } else {
-          if (!opaque(anc_ready)) {  // warp-uniform: t, half and plen are the same in every lane
-            anc = ancestors(p.parent + (size_t)s.b * n, n, node, valid, lane);
-            anc_ready = true;
-          }
           const uint32_t vis = (uint32_t)visible_keys(anc, key0 - plen);
 #pragma unroll
           for (int k = 0; k < 16; ++k)
