@@ -84,13 +84,17 @@ __device__ __forceinline__ void pair_sync(int quarter) {
 // the 64 levels a tree of at most 64 nodes can have.  Two coalesced loads and
 // shuffles replace one dependent global load per tree level.  Warp-collective;
 // a lane with want == false gets 0.
-__device__ inline uint64_t ancestors(const int* parent, int n, int node, bool want, int lane) {
+// The loads (parents_of) may be issued well before.
+__device__ __forceinline__ int2 parents_of(const int* parent, int n, int lane) {
+  return make_int2(lane < n ? parent[lane] : -1, lane + 32 < n ? parent[lane + 32] : -1);
+}
+__device__ inline uint64_t ancestors(int2 parents, int n, int node, bool want, int lane) {
   uint64_t a[2];
   int q[2];
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     const int x = lane + 32 * k;
-    const int px = x < n ? parent[x] : -1;
+    const int px = k == 0 ? parents.x : parents.y;
     a[k] = x < n ? 1ull << x : 0ull;
     q[k] = (px >= 0 && px < x) ? px : -1;
   }
@@ -115,6 +119,25 @@ __device__ inline uint64_t ancestors(const int* parent, int n, int node, bool wa
   const int v = want ? node : 0;
   const uint64_t r0 = __shfl_sync(0xffffffffu, a[0], v & 31), r1 = __shfl_sync(0xffffffffu, a[1], v & 31);
   return want ? (v < 32 ? r0 : r1) : 0ull;
+}
+
+// The share range of every slab that lies in several shares, for the merge kernel
+// ((-1, -1): written out directly, or no keys): slabs i, i + step, ...
+__device__ __forceinline__ void write_ranges(const BatchTiles& bt, int B, int H, int G, int weight, int2* ranges, int i,
+                                             int step) {
+  CostPartition P;
+  P.init(bt, B, H, G, weight);
+#pragma unroll 1
+  for (int bh = i; bh < B * H; bh += step) {
+    const int b = bh / H, nt = bt.ntiles[b];
+    int2 r = make_int2(-1, -1);
+    if (nt > 0) {
+      const long long first = bt.start[b] + (long long)(bh - b * H) * nt;
+      const int cf = P.cta_of(first), cl = P.cta_of(first + nt - 1);
+      if (cf != cl) r = make_int2(cf, cl);
+    }
+    ranges[bh] = r;
+  }
 }
 
 // Zeros for the sequences without cached keys (a prefix-only call's empty
@@ -153,13 +176,19 @@ __global__ void __launch_bounds__(kMergeWarps * 32) tree_merge_kernel(const int2
   // The next kernel may be scheduled now, onto the SMs this small grid leaves
   // free; it waits for this merge to complete before it touches memory.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  pdl_wait();  // the partials and ranges of the verification kernel are complete
   const int lane = threadIdx.x & 31;
-  const long long total = (long long)BH * rows;
-  for (long long wr = (long long)blockIdx.x * kMergeWarps + (threadIdx.x >> 5); wr < total;
-       wr += (long long)gridDim.x * kMergeWarps) {
-    const int bh = (int)(wr / rows), r = (int)(wr - (long long)bh * rows);
-    const int2 rg = ranges[bh];
+  const unsigned total = (unsigned)BH * (unsigned)rows, step = gridDim.x * kMergeWarps;
+  // Where a row's results come from and go to is known before the verification
+  // kernel has ended; after it, a row is two dependent loads and a store away.
+  bool waited = false;
+#pragma unroll 1
+  for (unsigned wr = blockIdx.x * kMergeWarps + (threadIdx.x >> 5); wr < total; wr += step) {
+    const int bh = (int)(wr / (unsigned)rows), r = (int)(wr - (unsigned)bh * (unsigned)rows);
+    const int b = bh / Hkv, h = bh - b * Hkv;
+    float* dst = out + out_row(b, h, r, rows, group, Hq) * D;
+    if (!waited) pdl_wait();  // the partials and ranges of the verification kernel are complete
+    waited = true;
+    const int2 rg = __ldcg(&ranges[bh]);
     if (rg.x < 0) continue;
     const size_t sstride = (size_t)rows * (D + 2);
     const float* row0 = partials + (size_t)(rg.x + bh) * sstride + (size_t)r * (D + 2);
@@ -201,8 +230,6 @@ __global__ void __launch_bounds__(kMergeWarps * 32) tree_merge_kernel(const int2
       M = Mg;
     }
     const float inv = L > 0.f ? 1.f / L : 0.f;
-    const int b = bh / Hkv, h = bh - b * Hkv;
-    float* dst = out + out_row(b, h, r, rows, group, Hq) * D;
 #pragma unroll
     for (int k = 0; k < kPairs; ++k)
       *reinterpret_cast<float2*>(dst + 64 * k + 2 * lane) = make_float2(acc[k].x * inv, acc[k].y * inv);

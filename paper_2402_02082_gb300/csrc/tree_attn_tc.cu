@@ -194,18 +194,20 @@ __global__ void __launch_bounds__(kThreads, 1)
     *abort_flag = 0;
     fence_barrier_init();
   }
-  pdl_wait();
-  if (warp == kMmaWarp) {
-    tc::tmem_alloc(tmem_slot, C::kTmemCols);
-    tc::tmem_relinquish();
-  }
-  tc::fence_before_sync();
   // this CTA: share x of the key sequence, row tile y of every slab in it;
   // shares of equal cost, a segment switch counted as seg_weight tiles
   const int G = gridDim.x / p.R, x = blockIdx.x / p.R, y = blockIdx.x - x * p.R;
   const int row0 = y * kM, rows_here = min(kM, p.rows - row0);
   const int weight = seg_weight(p.rows < kM ? p.rows : kM);
-  if (warp == 0) build_share(bt, p.kv_len, p.B, p.Hkv, p.max_kv_len, p.tree ? n : 0, kTK, G, weight, x, share);
+  if (warp == 0)
+    wait_and_build_share(bt, p.kv_len, p.B, p.Hkv, p.max_kv_len, p.tree ? n : 0, kTK, G, weight, x, share);
+  else
+    pdl_wait();
+  if (warp == kMmaWarp) {
+    tc::tmem_alloc(tmem_slot, C::kTmemCols);
+    tc::tmem_relinquish();
+  }
+  tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = *tmem_slot;
@@ -253,6 +255,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp >= kMmaWarp) {  // warps 9-11
     // ----------------------------------------------------------- MMA issue
     const int role = warp - kMmaWarp;  // 0, 1: S of tiles with j % 2 == role; 2: P.V
+    // The P.V warp has time until the first probabilities.
+    if (role == 2 && y == 0) write_ranges(bt, p.B, p.Hkv, G, weight, p.ranges, x * 32 + lane, G * 32);
+    __syncwarp();
     if (lane == 0) {
       // Ring positions are counted, not divided out.
       bool ok = true;
@@ -370,28 +375,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars[B_QFULL + (sg & 1)]);
     };
-    // The first segment's queries first: the first S products wait for them.
-    if (half == 0 && s.any()) write_q(s, 0);
-    // Then, off the path to the first S products: the share range of every
-    // slab split over several shares, for the merge kernel ((-1, -1): written
-    // out directly, or no keys), and zeros for a prefix-only call's sequences
-    // without cached keys (an empty softmax).
+    // The first segment's queries first: the first S products wait for them.  The
+    // parents its mask needs are loaded beside them.
     constexpr int kST = kSoftWarps * 32;
-    if (y == 0) {
-      CostPartition P;
-      P.init(bt, p.B, p.Hkv, G, weight);
-#pragma unroll 1
-      for (int bh = x * kST + (int)threadIdx.x; bh < p.B * p.Hkv; bh += G * kST) {
-        const int b = bh / p.Hkv, nt = bt.ntiles[b];
-        int2 r = make_int2(-1, -1);
-        if (nt > 0) {
-          const long long first = bt.start[b] + (long long)(bh - b * p.Hkv) * nt;
-          const int cf = P.cta_of(first), cl = P.cta_of(first + nt - 1);
-          if (cf != cl) r = make_int2(cf, cl);
-        }
-        p.ranges[bh] = r;
-      }
-    }
+    auto tree_keys = [&](const SegWalk& sq) { return p.tree && sq.t1 * kTK > bt.plen[sq.b]; };
+    int2 parents = make_int2(-1, -1);
+    if (s.any() && tree_keys(s)) parents = parents_of(p.parent + (size_t)s.b * n, n, lane);
+    if (half == 0 && s.any()) write_q(s, 0);
+    // Then, off the path to the first S products: zeros for a prefix-only call's
+    // sequences without cached keys (an empty softmax).
     if (!p.tree) zero_empty(bt, p.B, (long long)n * p.H * D, p.out, (int)blockIdx.x * kST + (int)threadIdx.x, (int)gridDim.x * kST);
     for (; s.any(); s.next(bt, p.Hkv), ++seg) {
       const int plen = bt.plen[s.b], len = bt.len[s.b];
@@ -400,7 +392,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       // the ancestor-or-self set of this row's tree node, if the segment has tree
       // keys, while its first keys are on their way
       uint64_t anc = 0;
-      if (p.tree && s.t1 * kTK > plen) anc = ancestors(p.parent + (size_t)s.b * n, n, node, valid, lane);
+      if (tree_keys(s)) {
+        if (seg > 0) parents = parents_of(p.parent + (size_t)s.b * n, n, lane);
+        anc = ancestors(parents, n, node, valid, lane);
+      }
 
       float m_used = -CUDART_INF_F, l = 0.f;  // l: this thread's share of the row sum
       // S of the next tile is loaded while this tile's exponentials run (within

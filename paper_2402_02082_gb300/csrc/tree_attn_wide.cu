@@ -189,16 +189,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     *abort_flag = 0;
     fence_barrier_init();
   }
-  pdl_wait();
+  // this CTA: share x of the key tiles, row tile y of every slab in it
+  const int G = gridDim.x / p.R, x = blockIdx.x / p.R, y = blockIdx.x - x * p.R;
+  const int row0 = y * kBM;
+  if (warp == 0)
+    wait_and_build_share(bt, p.kv_len, p.B, p.Hkv, p.max_kv_len, p.tree ? p.n : 0, kBN, G, kSegWeight, x, share);
+  else
+    pdl_wait();
   if (warp == kSWarp) {
     tc::tmem_alloc(tmem_slot, kTmemCols);
     tc::tmem_relinquish();
   }
   tc::fence_before_sync();
-  // this CTA: share x of the key tiles, row tile y of every slab in it
-  const int G = gridDim.x / p.R, x = blockIdx.x / p.R, y = blockIdx.x - x * p.R;
-  const int row0 = y * kBM;
-  if (warp == 0) build_share(bt, p.kv_len, p.B, p.Hkv, p.max_kv_len, p.tree ? p.n : 0, kBN, G, kSegWeight, x, share);
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = *tmem_slot;
@@ -258,6 +260,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_drain(&full[j % depth], (j / depth) & 1);
   } else if (warp == kSWarp || warp == kPVWarp) {
     // ----------------------------------------------------------- MMA issue
+    // The P.V warp has time until the first probabilities.
+    if (warp == kPVWarp && y == 0) write_ranges(bt, p.B, p.Hkv, G, kSegWeight, p.ranges, x * 32 + lane, G * 32);
+    __syncwarp();
     // Ring positions are counted, not divided out.
     if (lane == 0) {
       bool ok = true;
@@ -372,25 +377,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     const OutMap om{p.group, p.H};
     bool dead = false;
 
-    // The share range of every slab split over several shares, for the merge
-    // kernel ((-1, -1): written out directly), and zeros for a prefix-only
-    // call's sequences without cached keys (an empty softmax).
+    // Zeros for a prefix-only call's sequences without cached keys (an empty softmax).
     constexpr int kST = kSoftWarps * 32;
-    if (y == 0) {
-      CostPartition P;
-      P.init(bt, p.B, p.Hkv, G, kSegWeight);
-#pragma unroll 1
-      for (int bh = x * kST + (int)threadIdx.x; bh < p.B * p.Hkv; bh += G * kST) {
-        const int b = bh / p.Hkv, nt = bt.ntiles[b];
-        int2 rg = make_int2(-1, -1);
-        if (nt > 0) {
-          const long long first = bt.start[b] + (long long)(bh - b * p.Hkv) * nt;
-          const int cf = P.cta_of(first), cl = P.cta_of(first + nt - 1);
-          if (cf != cl) rg = make_int2(cf, cl);
-        }
-        p.ranges[bh] = rg;
-      }
-    }
     if (!p.tree)
       zero_empty(bt, p.B, (long long)p.n * p.H * D, p.out, (int)blockIdx.x * kST + (int)threadIdx.x,
                  (int)gridDim.x * kST);
@@ -399,10 +387,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (; s.any(); s.next(bt, p.Hkv)) {
       const int plen = bt.plen[s.b], nt = s.t1 - s.t0;
       const unsigned jl = i + nt - 1;  // the segment's last tile
-      // this row's node's ancestor-or-self set, found at the first tile that
-      // reaches the tree keys (prefix only: no tree keys)
+      // this row's node's ancestor-or-self set, if this group has a tile with tree
+      // keys, while the segment's first scores are on their way
       uint64_t anc = 0;
-      bool anc_ready = !p.tree;
+      int t_tree = plen / kBN - s.t0;  // the segment's first tile with tree keys
+      t_tree = t_tree < 0 ? 0 : t_tree;
+      t_tree += (int)((i + t_tree) ^ grp) & 1;
+      if (p.tree && t_tree < nt)
+        anc = ancestors(parents_of(p.parent + (size_t)s.b * p.n, p.n, lane), p.n, node, valid, lane);
       float m_own = -CUDART_INF_F, l = 0.f;  // the sum over this group's tiles and the reference it is taken against
       for (int t = (int)((i ^ grp) & 1u); t < nt; t += 2) {
         const unsigned j = i + t, bi = j % kSBufs;
@@ -413,10 +405,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         // lies past the tree): -inf, written back to the S buffer
         const int k0 = (s.t0 + t) * kBN - plen;  // the tile's first key, past the prefix
         if (k0 + kBN > 0) {
-          if (!opaque(anc_ready)) {
-            anc = ancestors(p.parent + (size_t)s.b * p.n, p.n, node, valid, lane);
-            anc_ready = true;
-          }
 #pragma unroll 1
           for (int c = 0; c < opaque(kBN / 32); ++c) {
             uint32_t o[32];
