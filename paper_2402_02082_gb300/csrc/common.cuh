@@ -433,8 +433,9 @@ __device__ inline void build_share(const BatchTiles& bt, const int* kv_len, int 
 // sequence's length is mostly the bound that the caller gave, so its table is
 // made from that while the previous kernel ends, and made again only if the
 // length turns out to be another: 1100 of the 2000 cycles from the wait to the
-// first copy (a call of 32 heads over 128 keys 10.9 -> 9.4 us with this and the ranges out of the softmax warps' way).  The lengths of
-// several sequences are rarely all the bound.
+// first copy (a call of 32 heads over 128 keys 10.9 -> 9.4 us with this and the
+// ranges out of the softmax warps' way).  The lengths of several sequences are
+// rarely all the bound.
 __device__ __forceinline__ void wait_and_build_share(const BatchTiles& bt, const int* kv_len, int B, int H, int max_kv_len,
                                                      int extra, int TK, int G, int w, int x, ShareStart* out) {
 #pragma unroll 1

@@ -199,10 +199,31 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int G = gridDim.x / p.R, x = blockIdx.x / p.R, y = blockIdx.x - x * p.R;
   const int row0 = y * kM, rows_here = min(kM, p.rows - row0);
   const int weight = seg_weight(p.rows < kM ? p.rows : kM);
-  if (warp == 0)
+  // one reader per tile: evict it first; R row tiles read each tile R times
+  const uint64_t kv_pol = p.R == 1 ? policy_evict_first() : policy_evict_normal();
+  auto load_tile = [&](const CUtensorMap* map, uint64_t* full, uint32_t dst, int row) {
+    mbar_arrive_expect_tx(full, C::kKVTile);
+    for (int hd = 0; hd < C::kHalves; ++hd)
+      tc::tma_load_2d(base + dst + hd * C::kKVHalf, map, hd * 64, row, full, kv_pol);
+  };
+  // The softmax threads' query row (see there), found before the wait: its node,
+  // and its place in a sequence's [node, head] rows of q and out.
+  const int rr = (lane >> 2) + 8 * (lane & 1), qi = rr * 4 + (warp & 3);
+  const bool valid = qi < rows_here;
+  int node = valid ? (row0 + qi) / p.group : 0;
+  int q_rel = node * p.H + (row0 + qi - node * p.group);
+  asm volatile("" : "+r"(node), "+r"(q_rel));
+  if (warp == 0) {
     wait_and_build_share(bt, p.kv_len, p.B, p.Hkv, p.max_kv_len, p.tree ? n : 0, kTK, G, weight, x, share);
-  else
+    if (lane == 0 && share->tiles > 0) {  // the first tile at once, not after the roles have found their way
+      const int row = (share->b * p.Hkv + share->h) * p.S_cap + share->t0 * kTK;
+      load_tile(&tmK, &bars[B_KFULL], C::off_K, row);
+      load_tile(&tmV, &bars[B_VFULL], off_V, row);
+    }
+    __syncwarp();
+  } else {
     pdl_wait();
+  }
   if (warp == kMmaWarp) {
     tc::tmem_alloc(tmem_slot, C::kTmemCols);
     tc::tmem_relinquish();
@@ -225,23 +246,20 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       const bool is_k = warp == kProdWarp;
       const CUtensorMap* map = is_k ? &tmK : &tmV;
-      tc::prefetch_tmap(map);
       uint64_t* full = &bars[is_k ? B_KFULL : B_VFULL];
       uint64_t* empty = &bars[is_k ? B_KEMPTY : B_VEMPTY];
       const uint32_t dst0 = is_k ? C::off_K : off_V;
-      // one reader per tile: evict it first; R row tiles read each tile R times
-      const uint64_t pol = p.R == 1 ? policy_evict_first() : policy_evict_normal();
       int issued = 0, st = 0;
       uint32_t phase = 1;
       bool ok = true;
       for (; s.any() && ok; s.next(bt, p.Hkv)) {
         int row = (s.b * p.Hkv + s.h) * p.S_cap + s.t0 * kTK;
         for (int t = s.t0; t < s.t1; ++t, row += kTK) {
-          ok = mbar_wait_small(&empty[st], phase, abort_flag);
-          if (!ok) break;
-          mbar_arrive_expect_tx(&full[st], C::kKVTile);
-          for (int hd = 0; hd < C::kHalves; ++hd)
-            tc::tma_load_2d(base + dst0 + st * C::kKVTile + hd * C::kKVHalf, map, hd * 64, row, &full[st], pol);
+          if (issued > 0) {  // the share's first tile is on its way already
+            ok = mbar_wait_small(&empty[st], phase, abort_flag);
+            if (!ok) break;
+            load_tile(map, &full[st], dst0 + st * C::kKVTile, row);
+          }
           ++issued;
           if (++st == ns) {
             st = 0;
@@ -337,12 +355,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     // w / 4 with the 16x64b TMEM shape: lane pair (t, t^2) shares one row,
     // thread t takes the row's even or odd columns (cpar), 16 of the 32 keys.
     const int quarter = warp & 3, half = warp >> 2;
-    const int rr = (lane >> 2) + 8 * (lane & 1);  // row within the quarter
+    // rr: row within the quarter; qi: the query row of this MMA row, within the row tile
     const int cpar = (lane >> 1) & 1;             // column parity of this thread
     const int row = quarter * 16 + rr;            // MMA row
-    const int qi = rr * 4 + quarter;              // the query row of this MMA row, within the row tile
-    const bool valid = qi < rows_here;
-    const int node = valid ? (row0 + qi) / p.group : 0;  // its tree node
     const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16);
     const uint32_t o_col = C::kTmemO + half * D;
     const int sid = threadIdx.x;                  // 0..255 among the softmax threads
@@ -353,10 +368,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     // Segment sg's queries into the swizzled Q tile (padding rows are zero);
     // the two threads of a row write chunks 0-3 and 4-7 of each 128-byte atom.
     // Key-half-0 warps only.
-    const OutMap om{p.group, p.H};
     // this thread's query row of the segment's slab in q / out (-1: none)
     auto row_at = [&](const SegWalk& sq) -> long long {
-      return valid ? om.row(sq.b, sq.h, row0 + qi, p.rows) : -1;
+      return valid ? (long long)sq.b * n * p.H + sq.h * p.group + q_rel : -1;
     };
     auto write_q = [&](const SegWalk& sq, int sg) {
       unsigned char* qrow = base + C::off_Q + (row >> 3) * 1024 + (row & 7) * 128;

@@ -192,10 +192,30 @@ __global__ void __launch_bounds__(kThreads, 1)
   // this CTA: share x of the key tiles, row tile y of every slab in it
   const int G = gridDim.x / p.R, x = blockIdx.x / p.R, y = blockIdx.x - x * p.R;
   const int row0 = y * kBM;
-  if (warp == 0)
+  // one reader per tile: evict it first; R row tiles read each tile R times
+  const uint64_t kv_pol = p.R == 1 ? policy_evict_first() : policy_evict_normal();
+  auto load_tile = [&](const CUtensorMap* map, uint64_t* full, unsigned char* dst, int row) {
+    mbar_arrive_expect_tx(full, C::kKV);
+    for (int hd = 0; hd < C::kHalves; ++hd) tc::tma_load_2d(dst + hd * kAtom, map, hd * 64, row, full, kv_pol);
+  };
+  auto load_q = [&](int b, int h) {
+    mbar_arrive_expect_tx(&bars[B_QFULL], C::kQBytes);
+    const int z = b * p.n + row0 / p.group;  // the row tile's first node in [B n, H, D]
+    for (int hd = 0; hd < C::kHalves; ++hd)
+      tc::tma_load_3d(base + C::off_Q + hd * kAtom, &tmQ, hd * 64, h * p.group, z, &bars[B_QFULL], policy_evict_first());
+  };
+  if (warp == 0) {
     wait_and_build_share(bt, p.kv_len, p.B, p.Hkv, p.max_kv_len, p.tree ? p.n : 0, kBN, G, kSegWeight, x, share);
-  else
+    if (lane == 0 && share->tiles > 0) {  // the first loads at once, not after the roles have found their way
+      const int row = (share->b * p.Hkv + share->h) * p.S_cap + share->t0 * kBN;
+      load_tile(&tmK, &bars[B_KFULL], base + C::off_K, row);
+      load_q(share->b, share->h);
+      load_tile(&tmV, &bars[B_VFULL], base + off_V, row);
+    }
+    __syncwarp();
+  } else {
     pdl_wait();
+  }
   if (warp == kSWarp) {
     tc::tmem_alloc(tmem_slot, kTmemCols);
     tc::tmem_relinquish();
@@ -211,10 +231,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ----------------------------------------------------------- producers
     // Warp 8 the keys, warp 11 the values: one loop, so that its code is there
     // once.  Lane 0 issues; the other lanes are there to clear the rows past a
-    // slab's last key in its last V tile.  One reader per tile: evict it first;
-    // R row tiles read each tile R times.
+    // slab's last key in its last V tile.
     const bool keys = warp == kKProdWarp;
-    const uint64_t pol = p.R == 1 ? policy_evict_first() : policy_evict_normal();
     const CUtensorMap* map = keys ? &tmK : &tmV;
     unsigned char* ring = base + (keys ? C::off_K : off_V);
     uint64_t* full = &bars[keys ? B_KFULL : B_VFULL];
@@ -230,11 +248,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         ok = warp_wait_small(&empty[st], phase, abort_flag);
         if (!ok) break;
         unsigned char* dst = ring + st * C::kKV;
-        if (lane == 0) {
-          mbar_arrive_expect_tx(&full[st], C::kKV);
-          for (int hd = 0; hd < C::kHalves; ++hd)
-            tc::tma_load_2d(dst + hd * kAtom, map, hd * 64, row, &full[st], pol);
-        }
+        if (lane == 0 && issued > 0) load_tile(map, &full[st], dst, row);  // the share's first tile is on its way already
         __syncwarp();
         ++issued;
         const int vrows = len - t * kBN;
@@ -275,16 +289,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         constexpr uint32_t idS = tc::idesc_bf16_f32(kBM, kBN, false, false);
         const uint64_t dQ = tc::sw128_desc(smem_u32(base + C::off_Q), 16, 1024);
         const uint64_t dK0 = tc::sw128_desc(smem_u32(base + C::off_K), 16, 1024);
-        const uint64_t pol_q = policy_evict_first();
         uint32_t b_phase = 1;
         bool q_loading = false;
         for (; s.any() && ok; s.next(bt, p.Hkv), ++seg) {
           if (seg > 0) ok = mbar_wait_small(&bars[B_QEMPTY], (seg - 1) & 1, abort_flag);
           if (!ok) break;
-          mbar_arrive_expect_tx(&bars[B_QFULL], C::kQBytes);
-          const int z = s.b * p.n + row0 / p.group;  // the row tile's first node in [B n, H, D]
-          for (int hd = 0; hd < C::kHalves; ++hd)
-            tc::tma_load_3d(base + C::off_Q + hd * kAtom, &tmQ, hd * 64, s.h * p.group, z, &bars[B_QFULL], pol_q);
+          if (seg > 0) load_q(s.b, s.h);
           q_loading = true;
           ok = mbar_wait_small(&bars[B_QFULL], seg & 1, abort_flag);
           if (ok) q_loading = false;
