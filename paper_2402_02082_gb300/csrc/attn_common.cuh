@@ -267,11 +267,4 @@ __device__ inline void combine_if_last(const Segment& s, int H, int nq, int r0, 
   consumer_sync(nthreads);
 }
 
-// Where query row r of slab (b, h) goes in the output: out_row with nq / group
-// nodes (tree verification and grouped-query cross-attention).
-struct OutMap {
-  int group, Hq;
-  __device__ long long row(int b, int h, int r, int nq) const { return (long long)out_row(b, h, r, nq, group, Hq); }
-};
-
 }  // namespace glide

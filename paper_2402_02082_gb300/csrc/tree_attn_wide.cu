@@ -83,6 +83,7 @@ constexpr int kBM = 128;          // query rows per row tile (MMA rows, TMEM lan
 constexpr int kBN = 128;          // keys per tile
 constexpr int kMaxStages = 4;     // K/V ring stages (the launch picks as many as fit)
 constexpr int kSoftWarps = 8;     // two groups of four: the even and the odd tiles
+constexpr int kFewRows = 24;      // a warp's rows up to which the epilogue stores them as they are (its comment)
 constexpr int kKProdWarp = 8;     // the K ring
 constexpr int kSWarp = 9;         // the queries and S
 constexpr int kPVWarp = 10;
@@ -384,7 +385,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int qrow = row0 + r;  // the slab's query row
     const bool valid = qrow < p.rows;
     const int node = valid ? qrow / p.group : 0;
-    const OutMap om{p.group, p.H};
+    const int q_rel = node * p.H + qrow - node * p.group;  // its place in a sequence's [node, head] rows of out
     bool dead = false;
 
     // Zeros for a prefix-only call's sequences without cached keys (an empty softmax).
@@ -521,32 +522,67 @@ __global__ void __launch_bounds__(kThreads, 1)
       pair_sync(quarter);  // read, before the next segment's reference goes in
       if (!dead) dead = !warp_wait_small(&bars[B_ODONE + (jl & 3)], (jl >> 2) & 1, abort_flag);
       tc::fence_after_sync();
-      uint32_t o[D / 2];
+      // Output rows of the whole slab in this share, else the share's partial [max,
+      // sum, o] (a partial row is 8-byte aligned).  A thread holds one row's columns;
+      // stored so, each 8 bytes of a warp's store lie in another sector, and 128 rows
+      // took 4400 cycles, 9900 on the last CTAs.  Eight lanes exchange their rows
+      // first, so that a store writes 64 consecutive bytes of four rows (32 / 8 heads:
+      // 4 x 2048 keys, 33 nodes 24.5 -> 19.6 us, 4 x 16384 63.1 -> 58.0).  A few rows
+      // are stored as they are (24: 11.5 us for 2048 keys, exchanged 11.8; 64: 13.5
+      // and 12.7).
+      const bool whole = s.whole(bt);
+      float* dst = whole ? p.out + ((long long)s.b * p.n * p.H + s.h * p.group) * D
+                         : partial_slot(p.partials, x + s.b * p.Hkv + s.h, p.rows, D) + 2;
+      const int rel = !valid || dead ? -1 : whole ? q_rel * D : qrow * (D + 2);
+      if (rel >= 0 && !whole && grp == 0) *reinterpret_cast<float2*>(dst + rel - 2) = make_float2(m_own, L);
+      const float scale = !whole ? 1.f : L > 0.f ? 1.f / L : 0.f;
+      const int warp_rows = p.rows - row0 - quarter * 32;
+      dst += grp * (D / 2);
+      auto load8 = [&](int c, float2 (&v)[8]) {
+        uint32_t o[16];
+        tc::tmem_ld16(lane_base + kTmemO + grp * (D / 2) + c * 16, o);
+        tc::tmem_wait_ld();
 #pragma unroll
-      for (int c = 0; c < D / 64; ++c)
-        tc::tmem_ld32(lane_base + kTmemO + grp * (D / 2) + c * 32, *reinterpret_cast<uint32_t(*)[32]>(o + 32 * c));
-      tc::tmem_wait_ld();
+        for (int k = 0; k < 8; ++k)
+          v[k] = make_float2(__uint_as_float(o[2 * k]) * scale, __uint_as_float(o[2 * k + 1]) * scale);
+      };
+      if (warp_rows > kFewRows) {
+        dst += 2 * (lane & 7);
+#pragma unroll 1
+        for (int c = 0; c < opaque(D / 32); ++c, dst += 16) {
+          float2 v[8];  // 8 x 8 pairs over 8 lanes, to be transposed
+          load8(c, v);
+#pragma unroll
+          for (int st = 4; st >= 1; st >>= 1)
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+              if (!(k & st)) {
+                const bool up = (lane & st) != 0;
+                const float2 send = up ? v[k] : v[k | st];
+                const float2 got =
+                    make_float2(__shfl_xor_sync(0xffffffffu, send.x, st), __shfl_xor_sync(0xffffffffu, send.y, st));
+                if (up) v[k] = got; else v[k | st] = got;
+              }
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const int to = __shfl_sync(0xffffffffu, rel, (lane & 24) + k);
+            if (to >= 0) *reinterpret_cast<float2*>(dst + to) = v[k];
+          }
+        }
+      } else if (warp_rows > 0) {
+        dst += rel;
+#pragma unroll 1
+        for (int c = 0; c < opaque(D / 32); ++c, dst += 16) {
+          float2 v[8];
+          load8(c, v);
+          if (rel >= 0)
+#pragma unroll
+            for (int k = 0; k < 8; ++k) *reinterpret_cast<float2*>(dst + 2 * k) = v[k];
+        }
+      }
       tc::fence_before_sync();
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars[B_OFREE]);
-      if (valid && !dead) {
-        if (s.whole(bt)) {  // the whole slab in this share: the output row
-          const float inv = L > 0.f ? 1.f / L : 0.f;
-          float* dst = p.out + om.row(s.b, s.h, qrow, p.rows) * D + grp * (D / 2);
-#pragma unroll
-          for (int e = 0; e < D / 2; e += 4)
-            *reinterpret_cast<float4*>(dst + e) =
-                make_float4(__uint_as_float(o[e]) * inv, __uint_as_float(o[e + 1]) * inv,
-                            __uint_as_float(o[e + 2]) * inv, __uint_as_float(o[e + 3]) * inv);
-        } else {  // the share's partial [max, sum, o] (a partial row is 8-byte aligned)
-          float* dst = partial_slot(p.partials, x + s.b * p.Hkv + s.h, p.rows, D) + (size_t)qrow * (D + 2);
-          if (grp == 0) *reinterpret_cast<float2*>(dst) = make_float2(m_own, L);
-#pragma unroll
-          for (int e = 0; e < D / 2; e += 2)
-            *reinterpret_cast<float2*>(dst + 2 + grp * (D / 2) + e) =
-                make_float2(__uint_as_float(o[e]), __uint_as_float(o[e + 1]));
-        }
-      }
       i += nt;
     }
   }
