@@ -52,22 +52,6 @@ __device__ __forceinline__ float transpose_reduce32(float (&part)[32], int lane)
   return part[0];
 }
 
-// The same for 16 keys: four exchange rounds and one final pairwise sum leave
-// lanes 2k and 2k+1 both holding the full sum for key k (16 shuffles).
-__device__ __forceinline__ float transpose_reduce16(float (&part)[16], int lane) {
-#pragma unroll
-  for (int off = 16, cnt = 8; off >= 2; off >>= 1, cnt >>= 1) {
-    const bool upper = (lane & off) != 0;
-#pragma unroll
-    for (int j = 0; j < cnt; ++j) {
-      const float send = upper ? part[j] : part[j + cnt];
-      const float keep = upper ? part[j + cnt] : part[j];
-      part[j] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-    }
-  }
-  return part[0] + __shfl_xor_sync(0xffffffffu, part[0], 1);
-}
-
 // ---------------------------------------------- lane-group mapping (cross)
 // The cross-attention consumers split a warp into 4 groups of 8 lanes: group
 // g takes keys 4g..4g+3 of a 16-key tile, and lane sub = lane & 7 owns the
