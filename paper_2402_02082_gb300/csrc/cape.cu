@@ -15,11 +15,11 @@
 // tokens, so the 8 largest keys of a row decide everything.
 //
 // One launch, no waiting:
-// 1. one CTA per chunk of kChunk probabilities of a row: every thread keeps a
-//    sorted top-8 of its elements in registers, a warp merges its lanes' lists
-//    with 8 rounds of "warp max, winner pops" (a 64-bit warp max is two
-//    redux.sync), warp 0 merges the warps' lists the same way and stores the
-//    chunk's top-8;
+// 1. one CTA per chunk of kChunk probabilities of a row: every thread sorts its
+//    eight keys (a 19-comparator network), a warp merges its lanes' lists with 8
+//    rounds of "warp max, winner pops" (a 64-bit warp max is two redux.sync), warp
+//    0 merges the warps' lists the same way, a list a lane, and stores the chunk's
+//    top-8;
 // 2. the CTA that completes a sequence's count (atomic counter over all of
 //    the sequence's chunks) merges each row's chunk lists (one warp per row)
 //    and builds the sequence's tree: the set sizes, the cap on verified
@@ -27,6 +27,10 @@
 // Publication is release/acquire: the chunk results are written, the writers
 // meet at a warp barrier, and one thread fences (acq_rel, gpu scope) and
 // counts; the completing CTA fences again before anyone reads them.
+//
+// What bounds it: the chain of a load, three merges, a fence and a count, and code
+// fetched on the way (insertion of every key into a list in registers made 65 KB
+// of it, this makes 34; 5 rows of 32000: 7.2 -> 6.9 us).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -39,7 +43,7 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kTop = 8;          // the proposal token + at most 7 expansion tokens
-constexpr int kChunk = 2048;     // probabilities per CTA (8 a thread: shorter insertion chains than 16)
+constexpr int kChunk = 2048;     // probabilities per CTA (8 a thread, one list)
 constexpr int kPerThread = kChunk / kThreads;
 static_assert(kPerThread % 4 == 0, "a thread's share is whole float4s");
 constexpr int kMaxPos = kMaxTree - 1;  // gamma <= max_tokens <= 63
@@ -103,19 +107,39 @@ __device__ __forceinline__ u64 warp_max_u64(u64 v) {
 
 __device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
-// Merges the 32 lanes' descending lists into the warp's top-8 (warp-uniform
-// result).  Keys are distinct except the zero filler, so one lane pops per round.
-__device__ __forceinline__ void warp_top(u64 (&t)[kTop], u64 (&out)[kTop]) {
-#pragma unroll
+// Merges the 32 lanes' descending lists: lane r < 8 gets the warp's r-th largest
+// key.  Keys are distinct except the zero filler, so one lane pops per round.
+__device__ __forceinline__ u64 warp_top(u64 (&t)[kTop], int lane) {
+  u64 mine = 0ull;
+#pragma unroll 1
   for (int r = 0; r < kTop; ++r) {
     const u64 m = warp_max_u64(t[0]);
-    out[r] = m;
+    if (lane == r) mine = m;
     if (t[0] == m) {
 #pragma unroll
       for (int j = 0; j < kTop - 1; ++j) t[j] = t[j + 1];
       t[kTop - 1] = 0ull;
     }
   }
+  return mine;
+}
+
+// Eight keys into descending order (Batcher's odd-even merge network).
+__device__ __forceinline__ void sort8(u64 (&t)[kTop]) {
+  auto order = [&](int i, int j) {
+    const u64 hi = t[i] > t[j] ? t[i] : t[j], lo = t[i] > t[j] ? t[j] : t[i];
+    t[i] = hi;
+    t[j] = lo;
+  };
+#pragma unroll
+  for (int p = 1; p < kTop; p <<= 1)
+#pragma unroll
+    for (int k = p; k >= 1; k >>= 1)
+#pragma unroll
+      for (int j = k % p; j + k < kTop; j += 2 * k)
+#pragma unroll
+        for (int i = 0; i < k; ++i)
+          if (i + j + k < kTop && (i + j) / (2 * p) == (i + j + k) / (2 * p)) order(i + j, i + j + k);
 }
 
 __global__ void __launch_bounds__(kThreads) cape_expand_kernel(const CapeParams p) {
@@ -143,59 +167,41 @@ __global__ void __launch_bounds__(kThreads) cape_expand_kernel(const CapeParams 
     const int lo = split * kChunk;
     const int hi = min(p.V, lo + kChunk);
     u64 t[kTop];
+    // all of this thread's loads first (one DRAM latency), then the keys
+    float x[kPerThread];
+    const bool vec = (p.V & 3) == 0;
+    if (vec) {
 #pragma unroll
-    for (int j = 0; j < kTop; ++j) t[j] = 0ull;
-    // all of this thread's loads first (one DRAM latency), then the inserts
-    if ((p.V & 3) == 0) {
-      const float4* v4 = reinterpret_cast<const float4*>(pr);
-      const int lo4 = lo / 4 + threadIdx.x, hi4 = hi / 4;
-      float4 x[kPerThread / 4];
-#pragma unroll
-      for (int u = 0; u < kPerThread / 4; ++u)
-        if (lo4 + u * kThreads < hi4) x[u] = __ldcs(v4 + lo4 + u * kThreads);
-#pragma unroll
-      for (int u = 0; u < kPerThread / 4; ++u) {
-        const int j = lo4 + u * kThreads;
-        if (j < hi4) {
-          top_insert(t, rank_key(x[u].x, 4 * j));
-          top_insert(t, rank_key(x[u].y, 4 * j + 1));
-          top_insert(t, rank_key(x[u].z, 4 * j + 2));
-          top_insert(t, rank_key(x[u].w, 4 * j + 3));
+      for (int u = 0; u < kPerThread; u += 4) {
+        const int j = lo + 4 * threadIdx.x + u * kThreads;
+        if (j < hi) {
+          const float4 f = __ldcs(reinterpret_cast<const float4*>(pr + j));
+          x[u] = f.x;
+          x[u + 1] = f.y;
+          x[u + 2] = f.z;
+          x[u + 3] = f.w;
         }
       }
     } else {
-      float x[kPerThread];
 #pragma unroll
       for (int u = 0; u < kPerThread; ++u)
         if (lo + threadIdx.x + u * kThreads < hi) x[u] = __ldcs(pr + lo + threadIdx.x + u * kThreads);
-#pragma unroll
-      for (int u = 0; u < kPerThread; ++u) {
-        const int j = lo + threadIdx.x + u * kThreads;
-        if (j < hi) top_insert(t, rank_key(x[u], j));
-      }
     }
-    u64 w[kTop];
-    warp_top(t, w);
-    if (lane == 0) {
 #pragma unroll
-      for (int j = 0; j < kTop; ++j) red[warp][j] = w[j];
+    for (int u = 0; u < kPerThread; ++u) {
+      const int j = vec ? lo + 4 * threadIdx.x + (u & ~3) * kThreads + (u & 3) : lo + threadIdx.x + u * kThreads;
+      t[u] = j < hi ? rank_key(x[u], j) : 0ull;
     }
+    sort8(t);
+    const u64 best = warp_top(t, lane);
+    if (lane < kTop) red[warp][lane] = best;
     __syncthreads();
     if (warp == 0) {
-      u64 c[kTop];
+      u64 c[kTop];  // lane w: warp w's list
 #pragma unroll
-      for (int j = 0; j < kTop; ++j) c[j] = 0ull;
-      for (int e = lane; e < kWarps * kTop; e += 32) top_insert(c, red[e / kTop][e % kTop]);
-      u64 ct[kTop];
-      warp_top(c, ct);
-      u64* slot = p.slots + ((size_t)row * p.splits + split) * kTop;
-      if (lane < kTop) {
-        u64 v = ct[0];
-#pragma unroll
-        for (int j = 1; j < kTop; ++j)
-          if (lane == j) v = ct[j];
-        __stcg(slot + lane, v);
-      }
+      for (int j = 0; j < kTop; ++j) c[j] = lane < kWarps ? red[lane][j] : 0ull;
+      const u64 of_chunk = warp_top(c, lane);
+      if (lane < kTop) __stcg(p.slots + ((size_t)row * p.splits + split) * kTop + lane, of_chunk);
       __syncwarp();
       if (lane == 0) {
         fence_acq_rel_gpu();   // release: the slot writes of this warp (seen through the barrier)
@@ -211,17 +217,19 @@ __global__ void __launch_bounds__(kThreads) cape_expand_kernel(const CapeParams 
   // ---- 2. this CTA completed sequence b: merge each row, one warp per row
   const int G = p.gamma;
   for (int i = warp; i < G; i += kWarps) {
-    u64 c[kTop];
+    u64 c[kTop];  // lane s: chunk s's list, merged with those of chunks s + 32, ...
+    const ulonglong2* lists = reinterpret_cast<const ulonglong2*>(p.slots + ((size_t)b * G + i) * p.splits * kTop);
 #pragma unroll
-    for (int j = 0; j < kTop; ++j) c[j] = 0ull;
-    const u64* slots = p.slots + ((size_t)b * G + i) * p.splits * kTop;
-    for (int e = lane; e < p.splits * kTop; e += 32) top_insert(c, __ldcg(slots + e));
-    u64 rt[kTop];
-    warp_top(c, rt);
-    if (lane == 0) {
-#pragma unroll
-      for (int j = 0; j < kTop; ++j) s_top[i][j] = rt[j];
+    for (int j = 0; j < kTop; j += 2) {
+      const ulonglong2 v = lane < p.splits ? __ldcg(lists + (lane * kTop + j) / 2) : make_ulonglong2(0ull, 0ull);
+      c[j] = v.x;
+      c[j + 1] = v.y;
     }
+#pragma unroll 1
+    for (int e = (lane + 32) * kTop; e < p.splits * kTop; e += (e + 1) % kTop ? 1 : 31 * kTop + 1)
+      top_insert(c, __ldcg(p.slots + ((size_t)b * G + i) * p.splits * kTop + e));
+    const u64 of_row = warp_top(c, lane);
+    if (lane < kTop) s_top[i][lane] = of_row;
   }
   __syncthreads();
 
