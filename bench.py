@@ -85,7 +85,7 @@ def kernel_source_hash(fname):
         return hashlib.sha256(f.read()).hexdigest()[:16]
 
 
-KERNEL_FILES = {"glide_cross_attn": "cross_attn.cu", "tree_verify_attn": "tree_attn_tc.cu",
+KERNEL_FILES = {"glide_cross_attn": "cross_direct.cu", "tree_verify_attn": "tree_attn_tc.cu",
                 "tree_accept": "accept.cu"}
 
 
