@@ -408,6 +408,39 @@ __device__ inline void build_share(const BatchTiles& bt, const int* kv_len, int 
     bt.sidx[0] = 0;
   }
   __syncwarp();
+  if (B <= 32) {
+    // The lookups of CostPartition::tile_at and of a tile's slab, lane b holding
+    // sequence b: ballots instead of searches through shared memory (8 x 40 heads,
+    // 512-4096 keys, 26 nodes 71.5 -> 71.2 us; 8 x 32 / 8 heads, 1024 keys, 16 nodes
+    // 16.9 -> 16.7).
+    const int nt = lane < B ? bt.ntiles[lane] : 0;
+    const int first = lane < B ? (int)bt.start[lane] : 0x7fffffff;
+    const int pos = lane < B ? first + w * bt.sidx[lane] : 0x7fffffff;
+    const int C = start + (slabs > 0 ? w * (slabs - 1) : 0), base = C / G, rem = C - base * G;
+    const int c = x + (lane & 1), v = c * base + (c < rem ? c : rem);
+    const unsigned m0 = __ballot_sync(0xffffffffu, pos <= __shfl_sync(0xffffffffu, v, 0));
+    const unsigned m1 = __ballot_sync(0xffffffffu, pos <= __shfl_sync(0xffffffffu, v, 1));
+    const int lo = 31 - __clz((lane & 1) ? m1 : m0);  // sequence 0 is at position 0
+    const int nl = __shfl_sync(0xffffffffu, nt, lo), fl = __shfl_sync(0xffffffffu, first, lo);
+    const int off = v - __shfl_sync(0xffffffffu, pos, lo);
+    int h = off / (nl + w);
+    if (h > H - 1) h = H - 1;
+    const int r = off - h * (nl + w);
+    const int g = v >= C ? start : fl + h * nl + (r < nl ? r : nl);
+    const int g0 = __shfl_sync(0xffffffffu, g, 0), g1 = __shfl_sync(0xffffffffu, g, 1);
+    const int b = 31 - __clz(__ballot_sync(0xffffffffu, first <= g0));
+    const int nb = __shfl_sync(0xffffffffu, nt, b), at = g0 - __shfl_sync(0xffffffffu, first, b);
+    if (lane == 0) {
+      ShareStart s = {0, 0, 0, g1 > g0 ? g1 - g0 : 0};
+      if (s.tiles > 0) {
+        s.b = b;
+        s.h = at / nb;
+        s.t0 = at - s.h * nb;
+      }
+      *out = s;
+    }
+    return;
+  }
   CostPartition P;
   P.init(bt, B, H, G, w);
   const int g = (int)P.tile_at(P.part_begin(x + (lane & 1)));
