@@ -175,6 +175,20 @@ def _cache_desc(q: torch.Tensor, K: torch.Tensor, V: torch.Tensor, scale, flags,
     return make_desc(B, H, D, S_cap, _dtype_code(K), scale, flags, max_ctas, H_kv=H_kv if H_kv != H else 0)
 
 
+def _check_lengths(kv_len: torch.Tensor, B: int, name: str = "kv_len"):
+    """The kernels read the first B values behind the tensor's pointer."""
+    if kv_len.dtype != torch.int32 or kv_len.numel() < B or not kv_len.is_contiguous():
+        raise TypeError(f"{name} must be contiguous int32 [B]")
+
+
+def _check_out(out: torch.Tensor, shape, what: str):
+    """The kernels write dense rows behind the tensor's pointer."""
+    if tuple(out.shape) != shape or not out.is_contiguous():
+        raise ValueError(f"{what} must be contiguous and of the stated shape")
+    if out.dtype != torch.float32:
+        raise TypeError("out must be fp32")
+
+
 def glide_cross_attn(q_draft: torch.Tensor, K_cache: torch.Tensor, V_cache: torch.Tensor, kv_len: torch.Tensor,
                      max_kv_len: int, out: torch.Tensor, workspace: torch.Tensor, scale: float = 0.0,
                      flags: int = 0, max_ctas: int = 0, stream=None) -> torch.Tensor:
@@ -186,10 +200,10 @@ def glide_cross_attn(q_draft: torch.Tensor, K_cache: torch.Tensor, V_cache: torc
     if st > 0:
         raise GlideError(st, "glide_cross_attn")
     desc = _cache_desc(q_draft, K_cache, V_cache, scale, flags, max_ctas)
-    if tuple(q_draft.shape) != (desc.B, 1, desc.H, desc.D) or tuple(out.shape) != (desc.B, 1, desc.H, desc.D):
-        raise ValueError("q_draft/out must be [B, 1, H, D]")
-    if out.dtype != torch.float32 or kv_len.dtype != torch.int32:
-        raise TypeError("out must be fp32 and kv_len int32")
+    if tuple(q_draft.shape) != (desc.B, 1, desc.H, desc.D):
+        raise ValueError("q_draft must be [B, 1, H, D]")
+    _check_out(out, (desc.B, 1, desc.H, desc.D), "out [B, 1, H, D]")
+    _check_lengths(kv_len, desc.B)
     st = lib().glide_cross_attn(ctypes.byref(desc), q_draft.data_ptr(), K_cache.data_ptr(), V_cache.data_ptr(),
                                 kv_len.data_ptr(), int(max_kv_len), out.data_ptr(), workspace.data_ptr(),
                                 workspace.numel() * workspace.element_size(), _stream(stream))
@@ -210,10 +224,10 @@ def glide_cross_attn_noalloc(q_draft: torch.Tensor, K_cache: torch.Tensor, V_cac
     if st > 0:
         raise GlideError(st, "glide_cross_attn_noalloc")
     desc = _cache_desc(q_draft, K_cache, V_cache, scale, flags, max_ctas)
-    if tuple(q_draft.shape) != (desc.B, 1, desc.H, desc.D) or tuple(out.shape) != (desc.B, 1, desc.H, desc.D):
-        raise ValueError("q_draft/out must be [B, 1, H, D]")
-    if out.dtype != torch.float32 or kv_len.dtype != torch.int32:
-        raise TypeError("out must be fp32 and kv_len int32")
+    if tuple(q_draft.shape) != (desc.B, 1, desc.H, desc.D):
+        raise ValueError("q_draft must be [B, 1, H, D]")
+    _check_out(out, (desc.B, 1, desc.H, desc.D), "out [B, 1, H, D]")
+    _check_lengths(kv_len, desc.B)
     st = lib().glide_cross_attn_noalloc(ctypes.byref(desc), q_draft.data_ptr(), K_cache.data_ptr(),
                                         V_cache.data_ptr(), kv_len.data_ptr(), int(max_kv_len), out.data_ptr(),
                                         _stream(stream))
@@ -233,10 +247,12 @@ def tree_verify_attn(q_tree: torch.Tensor, parent_idx: torch.Tensor, K_cache: to
         raise GlideError(st, "tree_verify_attn")
     desc = _cache_desc(q_tree, K_cache, V_cache, scale, flags, max_ctas)
     n = q_tree.shape[1]
-    if tuple(q_tree.shape) != (desc.B, n, desc.H, desc.D) or tuple(out.shape) != (desc.B, n, desc.H, desc.D):
-        raise ValueError("q_tree/out must be [B, n, H, D]")
-    if tuple(parent_idx.shape) != (desc.B, n) or parent_idx.dtype != torch.int32 or kv_len.dtype != torch.int32:
-        raise TypeError("parent_idx must be int32 [B, n] and kv_len int32 [B]")
+    if tuple(q_tree.shape) != (desc.B, n, desc.H, desc.D):
+        raise ValueError("q_tree must be [B, n, H, D]")
+    _check_out(out, (desc.B, n, desc.H, desc.D), "out [B, n, H, D]")
+    if tuple(parent_idx.shape) != (desc.B, n) or parent_idx.dtype != torch.int32 or not parent_idx.is_contiguous():
+        raise TypeError("parent_idx must be contiguous int32 [B, n]")
+    _check_lengths(kv_len, desc.B)
     st = lib().tree_verify_attn(ctypes.byref(desc), q_tree.data_ptr(), n, parent_idx.data_ptr(),
                                 K_cache.data_ptr(), V_cache.data_ptr(), kv_len.data_ptr(), int(max_kv_len),
                                 out.data_ptr(), workspace.data_ptr(), workspace.numel() * workspace.element_size(),
@@ -379,8 +395,9 @@ def glide_block_cross_attn(q: torch.Tensor, K_cache: torch.Tensor, V_cache: torc
     T = q.shape[1]
     if tuple(out.shape) != tuple(q.shape) or out.dtype != torch.float32 or not out.is_contiguous():
         raise ValueError("out must be contiguous fp32 [B, T, H, D]")
-    if seq_len.dtype != torch.int32 or tuple(seq_len.shape) != (desc.B,):
-        raise TypeError("seq_len must be int32 [B]")
+    if tuple(seq_len.shape) != (desc.B,):
+        raise TypeError("seq_len must be contiguous int32 [B]")
+    _check_lengths(seq_len, desc.B, "seq_len")
     st = lib().glide_block_cross_attn(ctypes.byref(desc), q.data_ptr(), T, int(L), K_cache.data_ptr(),
                                       V_cache.data_ptr(), seq_len.data_ptr(), out.data_ptr(), workspace.data_ptr(),
                                       workspace.numel() * workspace.element_size(), _stream(stream))

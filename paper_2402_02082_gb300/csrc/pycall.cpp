@@ -144,6 +144,11 @@ glide_attn_desc describe(const at::Tensor& q, const at::Tensor& K, const at::Ten
   d.H_kv = dim(K, 1) == d.H ? 0 : dim(K, 1);
   return d;
 }
+// What the kernels read and write as dense rows behind the pointer: the result, of the queries'
+// shape, and the lengths of d.B sequences.
+void check_dense(const at::Tensor& out, const at::Tensor& q, const at::Tensor& len, const glide_attn_desc& d) {
+  if (out.sizes() != q.sizes() || !out.is_contiguous() || len.numel() < d.B || !len.is_contiguous()) throw NotTaken{};
+}
 void options(glide_attn_desc& d, Args& a) {
   d.scale = a.f32();
   d.flags = a.u32();
@@ -159,7 +164,8 @@ PyObject* cross_attn(PyObject*, PyObject* const* v, Py_ssize_t n) {
     glide_attn_desc d = describe(q, K, V);
     const int32_t most = a.i32();
     const at::Tensor& out = a.tensor(at::kFloat);
-    if (q.size(1) != 1 || out.sizes() != q.sizes()) throw NotTaken{};
+    if (q.size(1) != 1) throw NotTaken{};
+    check_dense(out, q, len, d);
     void* ws = nullptr;
     size_t bytes = 0;
     if constexpr (!kNoAlloc) {
@@ -188,8 +194,9 @@ PyObject* verify_attn(PyObject*, PyObject* const* v, Py_ssize_t n) {
     glide_attn_desc d = describe(q, K, V);
     const int32_t most = a.i32(), nodes = dim(q, 1);
     const at::Tensor &out = a.tensor(at::kFloat), &w = a.any_tensor();
-    if (out.sizes() != q.sizes() || parent.dim() != 2 || parent.size(0) != d.B || parent.size(1) != nodes)
+    if (parent.dim() != 2 || parent.size(0) != d.B || parent.size(1) != nodes || !parent.is_contiguous())
       throw NotTaken{};
+    check_dense(out, q, len, d);
     options(d, a);
     const glide_stream_t stream = a.stream();
     const void *pq = q.data_ptr(), *pk = K.data_ptr(), *pv = V.data_ptr();
@@ -210,7 +217,8 @@ PyObject* block_attn(PyObject*, PyObject* const* v, Py_ssize_t n) {
     glide_attn_desc d = describe(q, K, V);
     const int32_t L = a.i32(), T = dim(q, 1);
     const at::Tensor &out = a.tensor(at::kFloat), &w = a.any_tensor();
-    if (out.sizes() != q.sizes() || !out.is_contiguous() || len.dim() != 1 || len.size(0) != d.B) throw NotTaken{};
+    if (len.dim() != 1 || len.size(0) != d.B) throw NotTaken{};
+    check_dense(out, q, len, d);
     d.scale = a.f32();
     d.max_ctas = a.i32();
     const glide_stream_t stream = a.stream();
