@@ -9,24 +9,6 @@
 #include "common.cuh"
 #include "kernels.h"
 
-namespace glide {
-
-int sm_count() {
-  static int cached_dev = -1;
-  static int cached = 0;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
-  if (dev != cached_dev) {
-    int v = 0;
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1) v = 1;
-    cached = v;
-    cached_dev = dev;
-  }
-  return cached;
-}
-
-}  // namespace glide
-
 namespace {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

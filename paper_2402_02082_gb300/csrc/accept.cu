@@ -38,6 +38,7 @@
 #include <stdint.h>
 
 #include "common.cuh"
+#include "device.h"
 #include "kernels.h"
 
 namespace glide {
@@ -429,15 +430,9 @@ size_t accept_workspace_bytes(int B, int n) {
 }
 
 cudaError_t launch_tree_accept(const AcceptArgs& a, cudaStream_t st) {
-  static int configured_dev = -1;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  static PerDevice<int> allowed;
+  const cudaError_t e = allow_smem(allowed, tree_accept_kernel, (int)kSmemBytes);
   if (e != cudaSuccess) return e;
-  if (configured_dev != dev) {
-    e = cudaFuncSetAttribute(tree_accept_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-    if (e != cudaSuccess) return e;
-    configured_dev = dev;
-  }
   AccParams p;
   p.draft = a.draft; p.parent = a.parent; p.logits = a.logits;
   p.path = a.path; p.len = a.len; p.bonus = a.bonus;

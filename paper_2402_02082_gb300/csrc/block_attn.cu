@@ -76,6 +76,7 @@
 #include <math_constants.h>
 
 #include "attn_common.cuh"
+#include "device.h"
 #include "kernels.h"
 #include "tc_attn.cuh"
 #include "tc_ptx.cuh"
@@ -701,13 +702,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 template <int D>
 cudaError_t launch_typed(const AttnArgs& a, cudaStream_t st) {
   using C = BlkCfg<D>;
-  static bool configured = false;
+  static PerDevice<int> allowed;
   const int limit = smem_optin_bytes();
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(block_attn_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  cudaError_t e = allow_smem(allowed, block_attn_kernel<D>, limit);
+  if (e != cudaSuccess) return e;
   if (C::kSmem > (size_t)limit) return cudaErrorNotSupported;
   CUtensorMap mq, mk, mv, mo;
   const long long kv_rows = (long long)a.B * a.Hkv * a.S_cap;

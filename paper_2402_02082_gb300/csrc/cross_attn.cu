@@ -42,6 +42,7 @@
 #include <math_constants.h>
 
 #include "attn_common.cuh"
+#include "device.h"
 #include "kernels.h"
 
 namespace glide {
@@ -435,13 +436,9 @@ template <typename T, int D>
 cudaError_t launch_typed(const AttnArgs& a, cudaStream_t st) {
   using C = CrossCfg<T, D>;
   const size_t smem = C::smem_bytes(a.B);
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(cross_attn_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)C::smem_bytes(kMaxBatch));
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static PerDevice<int> allowed;
+  cudaError_t e = allow_smem(allowed, cross_attn_kernel<T, D>, (int)C::smem_bytes(kMaxBatch));
+  if (e != cudaSuccess) return e;
   const long long tiles_ub = (long long)a.B * a.H * ((a.max_kv_len + kTK - 1) / kTK);
   long long G = a.max_ctas > 0 ? a.max_ctas : sm_count();
   if (G > kMaxCtas) G = kMaxCtas;
@@ -460,7 +457,7 @@ cudaError_t launch_typed(const AttnArgs& a, cudaStream_t st) {
   int levels = (int)(kMaxCtas / G);
   p.levels = levels > kLevels ? kLevels : (levels < 1 ? 1 : levels);
   p.scale_log2 = a.scale * kLog2e;
-  cudaError_t e = launch_pdl(cross_attn_kernel<T, D>, dim3((unsigned)G), dim3(kThreads), smem, st, p);
+  e = launch_pdl(cross_attn_kernel<T, D>, dim3((unsigned)G), dim3(kThreads), smem, st, p);
   if (e != cudaSuccess) return e;
   // The merge, also a programmatic dependent: it may be scheduled while the
   // attention kernel drains and waits (griddepcontrol.wait) until that kernel

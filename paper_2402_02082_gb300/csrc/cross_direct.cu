@@ -27,6 +27,7 @@
 
 #include "attn_common.cuh"
 #include "common.cuh"
+#include "device.h"
 #include "kernels.h"
 
 namespace glide {

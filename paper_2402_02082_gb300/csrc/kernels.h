@@ -83,8 +83,6 @@ struct SampleArgs {
   void* ws;
 };
 
-int sm_count();  // multiprocessors of the current device (cached per device)
-
 cudaError_t launch_cross_attn(const AttnArgs& a, cudaStream_t st);
 // Multi-head cross-attention without a workspace; cudaErrorNotSupported where
 // the streaming kernel of launch_cross_attn is the one to take.

@@ -20,6 +20,7 @@
 #include <stdint.h>
 
 #include "common.cuh"
+#include "device.h"
 #include "kernels.h"
 
 namespace glide {

@@ -33,9 +33,8 @@
 #include <math_constants.h>
 #include <stdint.h>
 
-#include <atomic>
-
 #include "attn_common.cuh"
+#include "device.h"
 #include "kernels.h"
 
 namespace glide {
@@ -366,24 +365,27 @@ cudaLaunchConfig_t config(int B, int C, cudaStream_t st, cudaLaunchAttribute* at
   return cfg;
 }
 
-// How many clusters of each size the chip runs at once (0: none, or unknown).
+// How many clusters of each size the current device runs at once (0: none).
 struct Room {
   int clusters[kMaxCluster + 1] = {};
 };
-Room find_room() {
-  Room r;
+cudaError_t find_room(Room& r) {
+  cudaError_t e = cudaFuncSetAttribute(spec_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)keep_bytes(1));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(spec_sample_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
   for (int C = 1; C <= kMaxCluster; ++C) {
     if (C > kPortable && C < kMaxCluster) continue;
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = config(1, C, nullptr, attr);
     cfg.attrs = attr + 1;  // the cluster's size alone
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&r.clusters[C], spec_sample_kernel, &cfg) != cudaSuccess) {
-      r.clusters[C] = 0;
-      cudaGetLastError();
-    }
+    e = cudaOccupancyMaxActiveClusters(&r.clusters[C], spec_sample_kernel, &cfg);
+    if (e == cudaSuccess) continue;
+    cudaGetLastError();
+    r.clusters[C] = 0;
+    if (e != cudaErrorInvalidClusterSize) return e;
   }
-  return r;
+  return cudaSuccess;
 }
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -397,22 +399,13 @@ size_t sample_workspace_bytes(int B, int gamma) {
 }
 
 cudaError_t launch_spec_sample(const SampleArgs& a, cudaStream_t st) {
-  static std::atomic<int> configured{-1};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (configured.load() != dev) {
-    e = cudaFuncSetAttribute(spec_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)keep_bytes(1));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(spec_sample_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    configured.store(dev);
-  }
+  static PerDevice<Room> rooms;
+  Room room;  // unknown: one CTA per sequence
+  if (rooms.get(room, find_room) != cudaSuccess) room = Room();
   // CTAs per sequence: as many as let all sequences run at once (a second wave
   // costs as much as the first: 16 sequences, gamma 4, C = 6 and 8: 10.2 and 13.3
   // us).  Sixteen only where they save a round of parts (4 sequences, gamma 8,
   // C = 8 and 16: 10.2 and 8.9 us; gamma 4: 7.95 and 8.1).
-  static const Room room = find_room();
   int C = kPortable;
   while (C > 1 && a.B > room.clusters[C]) --C;
   if (C == kPortable && (a.gamma + 1) * kParts > C * kWarps && a.B <= room.clusters[kMaxCluster]) C = kMaxCluster;

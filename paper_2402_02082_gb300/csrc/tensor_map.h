@@ -1,5 +1,4 @@
-// Host-side helpers for 2-D and 3-D TMA tensor maps and the launch's shared-memory
-// budget, shared by the tensor-core kernels.
+// Host-side helpers for 2-D and 3-D TMA tensor maps, shared by the tensor-core kernels.
 #pragma once
 
 #include <cuda.h>
@@ -72,19 +71,6 @@ inline bool make_f32_seq_map(CUtensorMap* m, void* base, long long B, long long 
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
          CUDA_SUCCESS;
-}
-
-// Largest dynamic shared memory a block of the current device may opt in to.
-inline int smem_optin_bytes() {
-  static int cached = -1;
-  if (cached < 0) {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
-      v = 227 * 1024;
-    cached = v;
-  }
-  return cached;
 }
 
 }  // namespace glide

@@ -20,6 +20,7 @@
 #include <math_constants.h>
 
 #include "attn_common.cuh"
+#include "device.h"
 #include "kernels.h"
 
 namespace glide {
@@ -261,13 +262,9 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_fma_kernel(const TreePa
 template <typename T, int D>
 cudaError_t launch_typed(const AttnArgs& a, cudaStream_t st) {
   using C = TreeCfg<T, D>;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(tree_attn_fma_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)C::smem_bytes(kMaxBatch));
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static PerDevice<int> allowed;
+  cudaError_t e = allow_smem(allowed, tree_attn_fma_kernel<T, D>, (int)C::smem_bytes(kMaxBatch));
+  if (e != cudaSuccess) return e;
   const long long tiles_ub = (long long)a.B * a.Hkv * ((a.max_kv_len + (a.tree ? a.nq : 0) + kTK - 1) / kTK);
   const int rows = a.nq * (a.H / a.Hkv);
   const int R = (rows + kRowTile - 1) / kRowTile;

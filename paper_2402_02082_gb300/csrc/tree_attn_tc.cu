@@ -73,6 +73,7 @@
 #include <math_constants.h>
 
 #include "attn_common.cuh"
+#include "device.h"
 #include "kernels.h"
 #include "tc_attn.cuh"
 #include "tc_ptx.cuh"
@@ -631,14 +632,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 template <int D>
 cudaError_t launch_typed(const AttnArgs& a, cudaStream_t st) {
   using C = TcCfg<D>;
-  static bool configured = false;
+  static PerDevice<int> allowed;
   const int limit = smem_optin_bytes();
-  if (!configured) {
-    cudaError_t e =
-        cudaFuncSetAttribute(tree_attn_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  cudaError_t e = allow_smem(allowed, tree_attn_tc_kernel<D>, limit);
+  if (e != cudaSuccess) return e;
   // As many K/V stages as the shared memory holds, and an even number: K slot
   // j % ns then only ever carries tiles of one parity, i.e. of one S issuer.
   const int group = a.H / a.Hkv;
@@ -668,7 +665,7 @@ cudaError_t launch_typed(const AttnArgs& a, cudaStream_t st) {
   p.Hkv = a.Hkv; p.group = group; p.rows = p.n * group; p.R = R; p.tree = a.tree;
   p.ns = ns;
   p.scale_log2 = a.scale * kLog2e;
-  cudaError_t e = launch_pdl(tree_attn_tc_kernel<D>, dim3((unsigned)(G * R)), dim3(kThreads), C::smem_bytes(a.B, ns),
+  e = launch_pdl(tree_attn_tc_kernel<D>, dim3((unsigned)(G * R)), dim3(kThreads), C::smem_bytes(a.B, ns),
                              st, mk, mv, p);
   if (e != cudaSuccess) return e;
   return launch_tree_merge<D>(p.ranges, p.partials, p.out, a.B * a.Hkv, p.rows, group, a.H, a.Hkv, st);

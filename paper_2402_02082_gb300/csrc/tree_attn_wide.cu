@@ -71,6 +71,7 @@
 #include <math_constants.h>
 
 #include "attn_common.cuh"
+#include "device.h"
 #include "kernels.h"
 #include "tc_attn.cuh"
 #include "tc_ptx.cuh"
@@ -601,13 +602,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 template <int D>
 cudaError_t launch_typed(const AttnArgs& a, cudaStream_t st) {
   using C = WideCfg<D>;
-  static bool configured = false;
+  static PerDevice<int> allowed;
   const int limit = smem_optin_bytes();
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(tree_attn_wide_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  cudaError_t e = allow_smem(allowed, tree_attn_wide_kernel<D>, limit);
+  if (e != cudaSuccess) return e;
   // As many stages as fit, the K ring first: S runs up to three tiles ahead of
   // P.V, so the keys are needed earlier than the values.
   int nk = kMaxStages, nv = kMaxStages;
@@ -646,7 +644,7 @@ cudaError_t launch_typed(const AttnArgs& a, cudaStream_t st) {
   if (G > kMaxCtas) G = kMaxCtas;
   if (G > tiles_ub) G = tiles_ub;
   if (G < 1) G = 1;
-  cudaError_t e = launch_pdl(tree_attn_wide_kernel<D>, dim3((unsigned)(G * p.R)), dim3(kThreads),
+  e = launch_pdl(tree_attn_wide_kernel<D>, dim3((unsigned)(G * p.R)), dim3(kThreads),
                              C::smem_bytes(a.B, nk, nv), st, mq, mk, mv, p);
   if (e != cudaSuccess) return e;
   return launch_tree_merge<D>(p.ranges, p.partials, p.out, a.B * a.Hkv, p.rows, group, a.H, a.Hkv, st);
