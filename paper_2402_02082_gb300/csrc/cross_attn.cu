@@ -3,9 +3,10 @@
 //   hd_j = SoftMax(Q^{m,j} (K^{l,j})^T / sqrt(d_k)) V^{l,j},
 // with no mask at inference.
 //
-// This is the streaming kernel: few (b, h) over long caches, fp32 clusters
-// that would not fit, and calls with a bound on the CTAs.  All other multi-head
-// calls take cross_direct.cu, which starts faster and streams as fast.
+// This is the streaming kernel: few (b, h) over long caches, fp32 batches whose
+// waves of clusters would cost more, and calls with a bound on the CTAs.  All
+// other multi-head calls take cross_direct.cu, which starts faster and, split as
+// it chooses there, streams at least as fast.
 //
 // The step reads every cached K and V byte once and does ~1 flop per byte, so
 // it is bound by HBM bandwidth.  Design:

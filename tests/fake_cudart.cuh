@@ -27,6 +27,7 @@ inline std::set<std::pair<const void*, int>> wide;        // (kernel, device) ->
 inline std::vector<Launch> launches;
 inline int attribute_calls = 0;
 
+inline cudaError_t last_error() { return cudaSuccess; }
 inline cudaError_t get_device(int* d) {
   *d = device;
   return cudaSuccess;
@@ -88,4 +89,4 @@ inline cudaError_t entry_point(const char*, void** p, unsigned, unsigned long lo
 #define cudaOccupancyMaxActiveClusters fake::max_clusters
 #define cudaLaunchKernelEx fake::launch
 #define cudaGetDriverEntryPointByVersion fake::entry_point
-#define cudaGetLastError() cudaSuccess
+#define cudaGetLastError fake::last_error
