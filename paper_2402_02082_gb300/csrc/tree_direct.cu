@@ -286,10 +286,22 @@ cudaError_t launch_tree_direct(const AttnArgs& a, cudaStream_t st) {
     }
   }
   const long long ctas = (long long)a.B * a.Hkv * ((rows + best_rows - 1) / best_rows) * best_C;
-  // One cluster's work over a very long cache leaves the chip idle (40000 keys,
-  // one row: here 40.1 us, the streaming kernel 37.2; two rows' clusters over
-  // 16384: 24.6 and 34.0).  It also honours a bound on the CTAs.
-  if (ctas <= kMaxCluster && keys > 32768) return cudaErrorNotSupported;
+  // Over a very long cache one or two slabs' clusters leave the chip idle, and the
+  // streaming kernel, which spreads the keys over all SMs, catches up with its
+  // later start (more than four rows of 64 floats: its merge takes longer).  Its
+  // time and this kernel's over long caches, as measured from 32000 to 100000 keys
+  // (us, this kernel / there, 65536 keys, D = 64: one slab, two rows 72.1 / 46.7,
+  // five rows 72.1 / 66.1, nine rows 71.6 / 107.4; two slabs, one row 76.7 / 62.9;
+  // four slabs 78.5 / 105.9; D = 128: one slab, two rows 80.0 / 59.6, two slabs, one
+  // row 86.0 / 81.9).
+  if (keys > 32768 && rows <= 8) {
+    const float slabs = (float)((long long)a.B * a.Hkv);
+    const float start = rows * a.D <= 256 ? 11.f + 13.f / slabs : 20.f + (a.D == 64 ? 22.f : 42.f) / slabs;
+    const float there = start + slabs * (float)keys * (a.D == 64 ? 0.00036f : 0.000485f);
+    const float here = best * ((a.D == 64 ? 1.13f : 1.28f) + 0.07f * slabs);
+    if (there < here) return cudaErrorNotSupported;
+  }
+  // The streaming kernel also honours a bound on the CTAs.
   if (a.max_ctas > 0 && ctas > a.max_ctas) return cudaErrorNotSupported;
   if (ctas > 0x7fffffffLL) return cudaErrorNotSupported;  // grid
   if (a.D == 128) return launch_d<128>(a, best_rows, best_C, st);
