@@ -160,9 +160,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 
 // The same wait in a fifth of the code (the kernels have some twenty of them,
 // and what does not fit the instruction cache is fetched again and again): on
-// giving up it only sets *abort, which must lie in shared memory, and the
-// kernel records the status once at its end (record_abort).
-__device__ __forceinline__ bool mbar_wait_small(uint64_t* bar, uint32_t parity, volatile int* abort) {
+// giving up (after limit_ns) it only sets *abort, which must lie in shared memory,
+// and the kernel records the status once at its end (record_abort).
+__device__ __forceinline__ bool mbar_wait_small(uint64_t* bar, uint32_t parity, volatile int* abort,
+                                                uint32_t limit_ns = (uint32_t)kWaitLimitNs) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\t.reg .u32 t0, t1;\n\t"
@@ -185,7 +186,7 @@ __device__ __forceinline__ bool mbar_wait_small(uint64_t* bar, uint32_t parity, 
       "mov.u32 %0, 0;\n"
       "DONE:\n\t}"
       : "=&r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity), "r"(smem_u32(const_cast<int*>(abort))), "n"((uint32_t)kWaitLimitNs)
+      : "r"(smem_u32(bar)), "r"(parity), "r"(smem_u32(const_cast<int*>(abort))), "r"(limit_ns)
       : "memory");
   return ok != 0;
 }
