@@ -23,6 +23,7 @@ import json
 import math
 import multiprocessing as mp
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -80,9 +81,19 @@ def measured_peaks():
 
 
 def kernel_source_hash(fname):
-    p = os.path.join(ROOT, "paper_2402_02082_gb300", "csrc", fname)
-    with open(p, "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()[:16]
+    """Over a kernel's file and the csrc headers it includes, directly or not."""
+    csrc = os.path.join(ROOT, "paper_2402_02082_gb300", "csrc")
+    seen, todo, h = set(), [fname], hashlib.sha256()
+    while todo:
+        f = todo.pop(0)
+        if f in seen or not os.path.exists(os.path.join(csrc, f)):
+            continue
+        seen.add(f)
+        with open(os.path.join(csrc, f), "rb") as src:
+            data = src.read()
+        h.update(data)
+        todo += re.findall(r'^#include "([^"]+)"', data.decode(), re.M)
+    return h.hexdigest()[:16]
 
 
 KERNEL_FILES = {"glide_cross_attn": "cross_direct.cu", "tree_verify_attn": "tree_attn_tc.cu",
@@ -261,10 +272,12 @@ def workload_config(w):
 
 
 # -------------------------------------------------------------------- main
-# kernels each library call launches at the bench workloads (verification: the
-# attention kernel and its split merge)
-LAUNCHES_PER_CALL = {"glide_cross_attn": 1, "tree_verify_attn": 2, "tree_accept": 1, "cape_expand": 1,
-                     "glide_kv_compact": 1}
+def launches_per_call(name, w, force_fma):
+    """Kernels that a library call launches at the bench workloads: one, but bf16 verification on the
+    tensor cores is the attention kernel and its split merge."""
+    return 2 if name == "tree_verify_attn" and w.dtype == "bf16" and not force_fma else 1
+
+
 CAPE_MAX_TOKENS = 32   # the cap on verified tokens of the paper's CaPE runs (Section 4)
 L2_BYTES = 129e6
 
@@ -1091,7 +1104,7 @@ def run_glide(args, rank, world, local_rank):
                 "next_rows": next_rows, "cpu_baseline": cpu_baseline,
                 "e2e": {"value": e2e_value, "unit": "GB/s", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                         "steps": e2e_steps, "launch": e2e_launch, "eager_value": e2e_eager},
-                "gpu_launches": sum(LAUNCHES_PER_CALL[nm] for nm in names) * args.steps, "clocks": clk}
+                "gpu_launches": sum(launches_per_call(nm, w, args.force_fma) for nm in names) * args.steps, "clocks": clk}
         if args.force_fma:
             line["config"]["tree_kernel"] = "cuda-core (forced)"
         print(json.dumps(line))
