@@ -212,10 +212,10 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 2 : 1) tree_direct_kernel(
     float pm[kMaxCluster], pl[kMaxCluster], po[kMaxCluster];
 #pragma unroll
     for (int c = 0; c < kMaxCluster; ++c) {
-      const uint32_t peer = c < p.C ? c : 0;
-      pm[c] = c < p.C ? load_peer(&part[r][0], peer) : -CUDART_INF_F;
-      pl[c] = load_peer(&part[r][1], peer);
-      po[c] = load_peer(&part[r][2 + d], peer);
+      // no CTA c: nothing, not CTA 0's values at weight 0 (0 times an infinity is a NaN)
+      pm[c] = c < p.C ? load_peer(&part[r][0], c) : -CUDART_INF_F;
+      pl[c] = c < p.C ? load_peer(&part[r][1], c) : 0.f;
+      po[c] = c < p.C ? load_peer(&part[r][2 + d], c) : 0.f;
       M = fmaxf(M, pm[c]);
     }
     const float ref = M == -CUDART_INF_F ? 0.f : M;
