@@ -16,11 +16,12 @@
 // ~1050 cycles; a softmax warp takes ~1500 on its 32 rows (S from TMEM, row
 // max, 128 exponentials a row, P back), a serial chain whatever runs beside
 // it.  Two softmax groups therefore take the tiles in turn, one thread per
-// position with its whole 128-key row: each has two tile periods for its chain,
-// and the pipe, not the chain, sets the pace (measured ~1400 cycles a tile; the
-// groups on the two key halves of every tile, meeting in a row-max exchange,
-// made ~2200).  The reference max of the online softmax passes from tile to
-// tile, so from group to group, through shared memory right after a tile's row
+// position with its whole 128-key row: each has two tile periods for its chain.
+// A tile takes ~1400 cycles (the groups on the two key halves of every tile,
+// meeting in a row-max exchange: ~2200): still the chain, with the round trips
+// of S and P between the roles, not the pipe, which is 54% busy over a call.  The
+// reference max of the online softmax passes from tile to tile, so from group to
+// group, through shared memory right after a tile's row
 // max is known; a group keeps its own row sum and takes it to the item's last
 // reference at the end.  P (bf16 pairs) overwrites the first 64 columns of its
 // S buffer.  S of tile i + 3 reuses the buffer of tile i, so it waits for the
@@ -40,8 +41,9 @@
 // 4 KB boxes of shared memory (the 128-byte swizzle) and writes them with bulk
 // tensor stores, which drain while the warps go on.
 //
-// Measured at B = 4, T = 2048, 32 heads, D = 128, L = 5: 139.6 -> 113.5 us, 65%
-// of the measured bf16 rate; B = 5, T = 1818, 32 over 8 heads, L = 4, ragged:
+// Measured at B = 4, T = 2048, 32 heads, D = 128, L = 5: 139.6 -> 112.7 us in
+// bursts of a few ms, 65% of the measured bf16 rate, 142.6 -> 122.2 us (60%)
+// sustained over a second; B = 5, T = 1818, 32 over 8 heads, L = 4, ragged:
 // 165.9 -> 127.4 us.  What is left: ~1500 cycles of every item's switch, waits
 // for K and V tiles that the other SMs' traffic delays, and CTAs with one pair
 // more than others.
@@ -124,8 +126,7 @@ struct BlkCfg {
   static constexpr uint32_t kStage = kEpiWarps * 2 * 4096;
   static constexpr uint32_t off_stg = off_Q + 2 * kQBytes;
   static constexpr uint32_t off_K = off_stg + kStage;
-  // The K ring, then the V ring, as many stages as fit: S runs up to three
-  // tiles ahead of P.V, so the keys get the deeper ring.  The depths are
+  // The K ring, then the V ring, as many stages as fit.  The depths are
   // compile-time constants: a division by a run-time depth costs an issuing
   // thread ~100 cycles each.
   static constexpr unsigned kNK = D == 128 ? 2 : 4, kNV = D == 128 ? 2 : 4;

@@ -240,8 +240,8 @@ __global__ void __launch_bounds__(kThreads, 1) spec_sample_kernel(const SamplePa
   const float inv = 1.f / st.y;
   const int seg = (V + kParts - 1) / kParts;  // contiguous tokens per segment
 
-  // Inverse-CDF draw from the current weights; -1 when they sum to 0.  Every
-  // warp of the cluster returns the same sign; the winning one the token.
+  // Inverse-CDF draw from the current weights: the warp with the winning segment
+  // writes the token.  False, in every warp of the cluster, when they sum to 0.
   auto draw = [&]() -> bool {
 #pragma unroll 1
     for (int sl = warp; rank + sl * p.C < kParts; sl += kWarps) {  // segments rank, rank + C, ... are this CTA's

@@ -54,7 +54,7 @@
 // and walked without divisions, ring positions are counted, waits are small and
 // the tree mask comes from one shifted window of the ancestor set, found before
 // the first scores; the thread that found the share issues its first copies: 92 KB
-// of code became 61 KB, batch-1 Vicuna-7B (2048 keys, 6 nodes) 17.7 -> 14.4 us,
+// of code became 65 KB, batch-1 Vicuna-7B (2048 keys, 6 nodes) 17.7 -> 14.4 us,
 // 1 x 32 heads over 128 keys 12.3 -> 9.4, the ragged Vicuna-13B batch (8 x 40
 // heads, 512-4096 keys, 26 nodes) 79.1 -> 71.7,
 // 3 x 40 heads of D = 64 with up to 441 keys 14.7 -> 12.1.  Long contexts, where

@@ -27,12 +27,13 @@
 //
 // Code size counts like a resource here (see the 64-row kernel): the loops are
 // rolled 64 scores at a time, the share is looked up once per CTA, waits are
-// small: 99 KB of code became 52 KB.  Measured on Mistral-7B's 32 over 8 heads
-// (16384 keys, 4 sequences): the 33-node tree, two row tiles (132 rows of 256),
-// 72.4 -> 62.7 us; the draft step, 4 rows, 48.1 -> 46.2; 2 sequences of 211
-// keys, one node, 11.2 -> 8.9; one sequence of 13645 keys, 3 nodes, 21.9 -> 18.7
-// (before: the groups on the two key halves of every tile, meeting in an
-// exchange of the row max).
+// small: 99 KB of code became 63 KB.  Measured on Mistral-7B's 32 over 8 heads
+// (16384 keys, 4 sequences), bursts of a few ms back to back: the 33-node tree,
+// two row tiles (132 rows of 256), 72.4 -> 57.6 us (62.7 before the epilogue's
+// exchange of rows; sustained over a second 74.0 -> 64.1); the draft step, 4 rows,
+// 48.1 -> 45.7; 2 sequences of 211 keys, one node, 11.2 -> 8.9; one sequence of
+// 13645 keys, 3 nodes, 21.9 -> 18.7 (before: the groups on the two key halves of
+// every tile, meeting in an exchange of the row max).
 //
 // Work: the slabs' 128-key tiles are cut into G shares of equal cost (a
 // segment switch counted as kSegWeight tiles), and R = ceil(rows / 128)
@@ -60,7 +61,7 @@
 // Masking: keys below the sequence's prefix length are visible to every row;
 // tree key c (at prefix + c) is visible to the rows of node i iff c is an
 // ancestor-or-self of i (the set built from the parent array by pointer
-// jumping, at the first tile that reaches the tree keys); keys past the
+// jumping, at the start of a segment that reaches the tree keys); keys past the
 // prefix and the n tree keys are masked, and their V rows are zeroed in
 // shared memory before P.V (the cache beyond them may hold anything).  In the
 // prefix-only mode a sequence without cached keys gets zeros.
