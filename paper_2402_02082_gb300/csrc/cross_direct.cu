@@ -262,7 +262,7 @@ int usual(long long slabs, long long slots, int keys) {
 // C is 5% cheaper, and the streaming kernel is taken where it is 3% cheaper than
 // that (fp32 only: its one CTA an SM leaves the start of every wave uncovered).
 //
-// The constants are fitted as a whole to 660 calls of each type and head size (8
+// The constants are fitted as a whole to some 650 calls of each type and head size (8
 // to 520 slabs, 384 to 16384 keys, equal and ragged, every C), over which the
 // choice is within 1 to 1.5% of the best C in the mean.  Streaming kernel /
 // `usual` / this (us; ragged: down to an eighth), bf16, D = 128: 3 x 52 heads, 8000
